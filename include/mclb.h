@@ -70,7 +70,9 @@ typedef enum {
 
 /* Which kernel schedule performs a timestep. */
 typedef enum {
-    MCLB_KERNEL_AUTO = 0,   /* the fused single-pass kernel                         */
+    MCLB_KERNEL_AUTO = 0,   /* the fused single-pass kernel, or on lattices too small to
+                               fill the GPU with it a kernel of small tiles (D2Q9, single
+                               handles): one launch per step, two with the Gibbs-Duhem form */
     MCLB_KERNEL_FUSED = 1,  /* stream, moments, potentials, force, collision in one
                                pass over the distributions, then a small launch that
                                refreshes the periodic ghost columns                 */
@@ -315,7 +317,8 @@ int mclb_conservation_rows(mclb_handle h, int y0, int nrows, double* mass, doubl
  * runs out (after about 2 s), the CTA returns, and mclb_status then reports
  * MCLB_ETIMEOUT.  The distributions are left unspecified: initialise again after
  * switching it off.  Steps are not replayed from CUDA graphs while it is on.  No effect
- * on the staged schedule.  Errors: EHANDLE. */
+ * on the staged schedule; a handle whose steps run by small tiles takes the single pass
+ * while it is on.  Errors: EHANDLE. */
 int mclb_test_withhold_copies(mclb_handle h, int on);
 
 /* HBM bytes one timestep must move at least: every stored value read once and
@@ -324,8 +327,9 @@ int mclb_test_withhold_copies(mclb_handle h, int on);
 double mclb_bytes_per_step(mclb_handle h);
 
 /* Kernel launches one timestep issues (2 for the fused schedule: the single pass and
- * the refresh of the periodic ghost columns; 3 for the staged; 1 on D1Q3, where one
- * launch advances a resident line by up to 4096 timesteps). */
+ * the refresh of the periodic ghost columns; 3 for the staged; 1 for the small tiles AUTO
+ * may pick, 2 with the Gibbs-Duhem form; 1 on D1Q3, where one launch advances a resident
+ * line by up to 4096 timesteps). */
 int mclb_launches_per_step(mclb_handle h);
 
 /* Release everything the handle owns.  NULL is accepted.  Synchronises. */

@@ -197,6 +197,7 @@ struct mclb_handle_s {
     Scratch sc;
     FusedPlan plan;
     bool fused;
+    TilePlan tile;                // the tile schedule's plan where AUTO picks it (ok = false otherwise)
     const LatticeTable* alt;      // D1Q3 and D3Q19 handles: their kernels (null for D2Q9)
     cudaStream_t stream;
     bool own_stream;
@@ -320,6 +321,8 @@ int make_tmap(mclb_handle h, int b)
 cudaError_t launch_one_step(mclb_handle h, int from)
 {
     const Problem& P = h->P;
+    if (h->tile.ok && !P.withhold)
+        return h->tab->step_tile(P, h->sc, h->tile, h->f[from], h->f[from ^ 1], h->stream);
     if (h->fused)
         return h->tab->step_fused(P, h->sc, h->plan, &h->tmap[from], &h->tmapr[from],
                                   &h->tmapw[from ^ 1], &h->tmapwr[from ^ 1], h->f[from],
@@ -512,6 +515,7 @@ int mclb_create(const mclb_params* params, mclb_handle* out)
         if (h->plan.ok && make_tmap(h, 0) == MCLB_OK && make_tmap(h, 1) == MCLB_OK) h->fused = true;
         if (!h->fused && h->kernel == MCLB_KERNEL_FUSED)
             return bail(fail(MCLB_EINVAL, "fused kernel unavailable for this problem"));
+        if (h->kernel == MCLB_KERNEL_AUTO && h->fused) h->tile = h->tab->plan_tile(P, sms);
     }
     cudaGetLastError();
     if (cudaStreamSynchronize(h->stream) != cudaSuccess)   // the zeroed buffers and status
@@ -673,6 +677,7 @@ int mclb_launches_per_step(mclb_handle h)
     if (check_handle(h)) return -1;
     if (h->P.lattice == MCLB_D1Q3) return 1;
     if (h->P.lattice == MCLB_D3Q19) return h->fused ? 2 : 3;   // density + march, or staged
+    if (h->tile.ok) return h->P.force_form == FORCE_GIBBS_DUHEM ? 2 : 1;
     if (h->fused) return h->P.walls ? 5 : 2;   // k_march, k_ghosts (+ three wall-row launches)
     return 3;
 }

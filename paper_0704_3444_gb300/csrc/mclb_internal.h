@@ -83,6 +83,16 @@ struct FusedPlan {
     bool ok;
 };
 
+// Launch plan of the tile schedules: k_tile (tile.cuh), tiles of (1 << lx) x ty sites, or k_rows
+// (rows.cuh, lx = 0).
+struct TilePlan {
+    int lx, ty;
+    int gx, gy;
+    int threads;
+    size_t smem;
+    bool ok;
+};
+
 // Kernels of a lattice other than the D2Q9 family -- D1Q3 (line3.cuh) or D3Q19 (cube.cuh)
 // -- for one storage type (FP64 and FP32 only).  Distributions: post-collision values
 // ([s][3][nx] for D1Q3, [s][z][y][19][x] for D3Q19); pre-collision f_i(r) = f*_i(r - v_i).
@@ -138,6 +148,10 @@ struct KernelTable {
                               const CUtensorMap* tmap_in, const CUtensorMap* tmapr_in,
                               const CUtensorMap* tmapw_out, const CUtensorMap* tmapwr_out,
                               const void* fin, void* fout, cudaStream_t st);
+    // one timestep fin -> fout by small tiles (one launch, two with the Gibbs-Duhem force)
+    TilePlan (*plan_tile)(const Problem&, int sm_count);
+    cudaError_t (*step_tile)(const Problem&, const Scratch&, const TilePlan&, const void* fin,
+                             void* fout, cudaStream_t st);
     // one staged timestep fin -> fout (three launches through scratch)
     cudaError_t (*step_staged)(const Problem&, const Scratch&, const void* fin, void* fout,
                                cudaStream_t st);

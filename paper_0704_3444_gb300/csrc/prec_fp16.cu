@@ -5,6 +5,7 @@
 namespace mclb {
 
 void fill_fp16_march(KernelTable& t);   // prec_fp16_march.cu
+void fill_fp16_tile(KernelTable& t);   // prec_fp16_tile.cu
 void fill_fp16_staged(KernelTable& t);   // prec_fp16_staged.cu
 void fill_fp16_batch(KernelTable& t);   // prec_fp16_batch.cu
 
@@ -14,6 +15,7 @@ const KernelTable& table_fp16()
         KernelTable x{};
         table_base<__half>(x, CU_TENSOR_MAP_DATA_TYPE_FLOAT16);
         fill_fp16_march(x);
+        fill_fp16_tile(x);
         fill_fp16_staged(x);
         fill_fp16_batch(x);
         return x;

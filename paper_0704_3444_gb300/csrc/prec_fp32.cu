@@ -5,6 +5,7 @@
 namespace mclb {
 
 void fill_fp32_march(KernelTable& t);   // prec_fp32_march.cu
+void fill_fp32_tile(KernelTable& t);   // prec_fp32_tile.cu
 void fill_fp32_staged(KernelTable& t);   // prec_fp32_staged.cu
 void fill_fp32_batch(KernelTable& t);   // prec_fp32_batch.cu
 void fill_fp32_line3(KernelTable& t);   // prec_fp32_line3.cu
@@ -16,6 +17,7 @@ const KernelTable& table_fp32()
         KernelTable x{};
         table_base<float>(x, CU_TENSOR_MAP_DATA_TYPE_FLOAT32);
         fill_fp32_march(x);
+        fill_fp32_tile(x);
         fill_fp32_staged(x);
         fill_fp32_batch(x);
         fill_fp32_line3(x);

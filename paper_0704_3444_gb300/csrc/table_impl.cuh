@@ -10,7 +10,9 @@
 #include "line3.cuh"
 #include "march.cuh"
 #include "mass.cuh"
+#include "rows.cuh"
 #include "staged.cuh"
+#include "tile.cuh"
 
 namespace mclb {
 
@@ -280,6 +282,112 @@ struct Launch {
         k_mass_apply<T><<<dim3(gx, P.N), MASS_THREADS, 0, st>>>((T*)f, v, sc.partial, sc.mass_ref,
                                                                 record);
         return cudaGetLastError();
+    }
+};
+
+// Launch with programmatic stream serialisation: the kernel may be scheduled while the one
+// before it drains (it waits for that one's end itself).
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st,
+                             A... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
+
+// The tile schedule (tile.cuh) for one storage type.
+template <typename T>
+struct TileLaunch {
+    using C = typename Storage<T>::C;
+
+    // Most sites x components for which a tile kernel beats the march (measured on both sides of
+    // each line, us per step, tile / march; between walls the march also pays three band
+    // launches, about 20 us):
+    //   FP64: it runs at the FP64 pipe's rate on every SM, and collide_poly needs fewer FP64
+    //     operations: 64 x 64 x 2 10.8 / 107, 1024^2 x 2 652 / 745, 2048^2 x 2 2589 / 2609; five
+    //     and more components 300 x 200 x 5 116 / 206, 1024^2 x 5 1819 / 1493
+    //   FP32 (k_rows): 1000^2 x 1 18.1 / 26.3; 700^2 x 2 20.5 / 22.3, 1024^2 x 2 38 / 37;
+    //     512 x 384 x 3 14.7 / 18.5, 700 x 600 x 3 29.8 / 25.7; 400^2 x 4 21.7 / 20.1;
+    //     300^2 x 5 13.5 / 19.4, 500 x 450 x 5 24.9 / 23.6; walls 1000 x 333 x 3 21 / 39,
+    //     1500 x 1200 x 3 107 / 95.  k_tile, six and more: 300^2 x 6 20.0 / 23.1
+    //   16-bit: 400 x 300 x 4 19.7 / 22.8, 400^2 x 5 33 / 30; walls 1000 x 700 x 3 65.5 / 66.6
+    //   Gibbs-Duhem: FP64 1024^2 x 3 1098 / 1131; FP32 300^2 x 2 10.4 / 16.0, 512 x 384 x 3
+    //     22.8 / 18.5
+    static long long most(const Problem& P)
+    {
+        const int N = P.N;
+        if (sizeof(C) == 8) return N >= 5 ? 1500000 : (P.force_form == FORCE_GIBBS_DUHEM ? 3000000 : 8000000);
+        if (P.force_form == FORCE_GIBBS_DUHEM) return 350000;
+        if (Storage<T>::shifted) return P.walls ? 2000000 : 600000;
+        if (P.walls) return 4000000;
+        return N == 1 ? 2000000 : N == 2 ? 1200000 : N == 4 || N >= 6 ? 550000 : 900000;
+    }
+
+    // FP32 above this goes to k_rows, below to k_tile (200 x 100 x 3 5.6 / 6.2 us, 300^2 x 2
+    // 7.7 / 7.3, 300^2 x 5 17 / 13.5)
+    static constexpr long long ROWS_LEAST = 150000;
+
+    static TilePlan plan(const Problem& P, int)
+    {
+        TilePlan pl{};
+        const bool gd = P.force_form == FORCE_GIBBS_DUHEM;
+        if (P.S * P.N > most(P)) return pl;
+        if constexpr (std::is_same<T, float>::value) {
+            if (!gd && P.S * P.N >= ROWS_LEAST && P.ny >= ROWS_MIN_NY && P.N <= ROWS_NMAX) {
+                pl.gx = (P.nx + ROWS_X - 1) / ROWS_X;
+                pl.gy = (P.ny + ROWS_Y - 1) / ROWS_Y;
+                pl.threads = 32 * ROWS_WPC * P.N;
+                pl.ok = pl.gy < 65536;
+                return pl;
+            }
+        }
+        // 16 x 8 sites; 8 x 4 where five and more components fill a CTA with fewer sites, and
+        // in FP64, whose few operations per clock and SM want every SM busy, below about 100
+        // of the larger tiles (100 x 90 x 2 11.4 us, 15.7 with 16 x 8; 160 x 96 x 2 21.2, 20.3)
+        const bool small = P.N >= 5 || (sizeof(C) == 8 && P.S < 12800);
+        const int ty = small ? 4 : 8;
+        pl.lx = small ? 3 : 4;
+        pl.ty = ty;
+        pl.gx = (P.nx + (1 << pl.lx) - 1) >> pl.lx;
+        pl.gy = (P.ny + ty - 1) / ty;
+        pl.threads = P.N * (ty << pl.lx);
+        pl.smem = sizeof(C) * tile_smem_values(P.N, 1 << pl.lx, ty, gd);
+        pl.ok = pl.threads <= tile_max_threads<T>() && pl.smem <= 48 * 1024 && pl.gy < 65536 &&
+                (long long)P.plane * P.N < (1LL << 31);
+        return pl;
+    }
+
+    static cudaError_t step(const Problem& P, const Scratch& sc, const TilePlan& pl, const void* fin,
+                            void* fout, cudaStream_t st)
+    {
+        const auto p = make_params<C>(P, sc.status);
+        const C* rs = nullptr;
+        if (P.force_form == FORCE_GIBBS_DUHEM) {
+            const cudaError_t e = launch_dependent(k_tile_rho<T>, dim3((unsigned)((P.S + 127) / 128), P.N),
+                                                   128, 0, st, (const T*)fin, (C*)sc.rho_s, p);
+            if (e != cudaSuccess) return e;
+            rs = (const C*)sc.rho_s;
+        }
+        if constexpr (std::is_same<T, float>::value) {
+            if (pl.lx == 0)
+                MCLB_DISPATCH_N(P.N, {
+                    return launch_dependent(P.walls ? k_rows<NN, true> : k_rows<NN, false>,
+                                            dim3(pl.gx, pl.gy), pl.threads, 0, st, (const T*)fin, (T*)fout, p);
+                });
+        }
+        MCLB_DISPATCH_N(P.N, {
+            return launch_dependent(k_tile<T, NN>, dim3(pl.gx, pl.gy), pl.threads, pl.smem, st,
+                                    (const T*)fin, (T*)fout, rs, p, pl.lx, pl.ty);
+        });
     }
 };
 
@@ -745,6 +853,14 @@ inline void fill_march(KernelTable& t)
 {
     t.plan_fused = &Launch<T>::plan_fused;
     t.step_fused = &Launch<T>::step_fused;
+}
+
+// single handles on D2Q9: small tiles
+template <typename T>
+inline void fill_tile(KernelTable& t)
+{
+    t.plan_tile = &TileLaunch<T>::plan;
+    t.step_tile = &TileLaunch<T>::step;
 }
 
 // single handles on D2Q9: the staged schedule and the diagnostics

@@ -1,0 +1,127 @@
+"""The tile schedules (one launch per timestep on lattices too small for the march), which AUTO
+picks by size: against the FP64 oracle at the edges of their tiles -- lattices smaller than a
+tile, exact multiples, remainders of one -- with every term on, between walls and under the
+Gibbs-Duhem form, and against the other schedules' ghost columns by bands."""
+import numpy as np
+import pytest
+
+import paper_0704_3444_gb300 as mclb
+from oracle import Oracle
+from paper_0704_3444_gb300 import inputs
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.fixture(scope="module", autouse=True)
+def built():
+    mclb.build()
+    mclb.load()
+
+
+def _pair(shape, precision, fv=0, walls=0, gd=0, amp=0.3, seed=70):
+    nx, ny, n = shape
+    rho, u = inputs.random_state(n, nx, ny, seed=seed + nx + n, amp=amp, umax=0.03)
+    chi = inputs.uniform_chi(n, 1.6)
+    kw = dict(m=[1.0 + (k % 3) for k in range(n)], theta=0.4, kappa=0.0 if gd else 0.02,
+              force=(1e-5, -2e-5), forcing_velocity=fv, walls=walls, force_form=gd)
+    sim = mclb.Simulation(n, nx, ny, 0.9, chi, precision=precision, **kw)
+    orc = Oracle(n, nx, ny, 0.9, chi, **kw)
+    sim.init_fields(rho, u)
+    orc.init(rho, u)
+    return sim, orc
+
+
+def _rel(a, b):
+    return np.max(np.abs(a - b)) / max(np.max(np.abs(b)), 1e-300)
+
+
+SHAPES = [(1, 1, 2), (4, 4, 2), (1, 9, 3), (9, 1, 1), (5, 3, 3), (8, 4, 5), (9, 5, 6), (33, 13, 8),
+          (130, 100, 4), (161, 97, 2)]
+
+
+@pytest.mark.parametrize("mode", ["periodic", "barycentric", "walls", "gibbs_duhem"])
+@pytest.mark.parametrize("shape", SHAPES, ids=lambda s: f"{s[0]}x{s[1]}N{s[2]}")
+def test_fp64_parity(shape, mode):
+    """40 FP64 steps (one graph of 32 and 8 more) to the oracle parity of the other
+    schedules (1e-12 of the field's max-norm)."""
+    gd = mode == "gibbs_duhem"
+    if gd and shape[2] > 3:
+        pytest.skip("the form runs staged there")
+    sim, orc = _pair(shape, "fp64", fv=int(mode != "periodic"), walls=int(mode == "walls"), gd=int(gd))
+    assert sim.launches_per_step == (2 if gd else 1)
+    sim.step(40)
+    assert orc.run(40) == 0
+    assert sim.status() == 0
+    assert _rel(sim.get_state(), orc.f) < 1e-12
+    # the ghost columns are the columns they repeat: a schedule that reads them goes on from
+    # the same stored rows
+    nx, ny, n = shape
+    if mode != "walls":
+        import torch
+        band = torch.empty(sim.rows_bytes(ny) // 8, dtype=torch.float64, device="cuda")
+        sim.pack_rows(0, ny, band)
+        fused = mclb.Simulation(n, nx, ny, 0.9, inputs.uniform_chi(n, 1.6), precision="fp64",
+                                kernel=mclb.KERNEL_FUSED, m=[1.0 + (k % 3) for k in range(n)], theta=0.4,
+                                kappa=0.0 if gd else 0.02, force=(1e-5, -2e-5),
+                                forcing_velocity=int(mode != "periodic"), force_form=int(gd))
+        torch.cuda.synchronize()
+        fused.unpack_rows(0, ny, band)
+        fused.step(3)
+        orc.run(3)
+        assert _rel(fused.get_state(), orc.f) < 1e-12
+        fused.close()
+    sim.close()
+
+
+@pytest.mark.parametrize("walls", [0, 1])
+@pytest.mark.parametrize("shape", [(37, 21, 3), (16, 8, 1), (400, 190, 2), (279, 181, 3), (29, 5600, 1), (420, 160, 4),
+                                   (225, 200, 5), (90, 70, 8)],
+                         ids=lambda s: f"{s[0]}x{s[1]}N{s[2]}")
+def test_fp32_parity(shape, walls):
+    """100 FP32 steps: rho, U and mu within the FP32 tolerance of the fields (1e-5)."""
+    sim, orc = _pair(shape, "fp32", walls=walls, amp=0.1)
+    assert sim.launches_per_step == 1
+    sim.step(100)
+    assert orc.run(100) == 0
+    assert sim.status() == 0
+    gm, om = sim.moments(), orc.moments()
+    for k in ("rho", "U", "mu"):
+        assert np.max(np.abs(gm[k] - om[k])) < 1e-5, k
+    sim.close()
+
+
+@pytest.mark.parametrize("precision", ["bf16", "fp16"])
+@pytest.mark.parametrize("shape,walls", [((37, 21, 3), 0), ((150, 61, 4), 1), ((16, 8, 6), 0)],
+                         ids=["37x21N3", "150x61N4walls", "16x8N6"])
+def test_16_bit_parity(shape, walls, precision):
+    """The 16-bit formats: densities within 2e-3 and every component's mass to 1e-6, as the
+    other schedules keep them."""
+    sim, orc = _pair(shape, precision, walls=walls, amp=0.1)
+    assert sim.launches_per_step == 1
+    m0 = sim.conservation()["mass"]
+    sim.step(50)
+    assert orc.run(50) == 0
+    assert sim.status() == 0
+    assert np.max(np.abs(sim.moments()["rho"] - orc.moments()["rho"])) < 2e-3
+    assert np.max(np.abs(sim.conservation()["mass"] / m0 - 1.0)) < 1e-6
+    sim.close()
+
+
+@pytest.mark.parametrize("precision,shape", [("fp64", (50, 40, 2)), ("fp32", (50, 40, 2)), ("fp32", (300, 190, 3))])
+def test_resume_and_non_finite(precision, shape):
+    """A state read back and set again goes on bitwise; a density that turns non-finite is
+    reported."""
+    sim, _ = _pair(shape, precision)
+    sim.step(35)
+    mid = sim.get_state()
+    sim.step(33)
+    end = sim.get_state()
+    sim.set_state(mid)
+    sim.step(33)
+    assert np.array_equal(sim.get_state(), end)
+    assert sim.status() == 0
+    mid[:] = -mid
+    sim.set_state(mid)
+    sim.step_nocheck(1)
+    assert sim.status() == -4
+    sim.close()
