@@ -12,11 +12,17 @@
 //     thread) and advances it by K steps in shared memory before writing it back, so a
 //     line crosses HBM once per launch instead of once per step.  A batch launches one
 //     CTA per line (every line of the same N in one launch).  Three CTA barriers per
-//     step, no other waits.
+//     step, no other waits.  FP64 lines whose N threads per site fit a cluster take
+//     k_line3_resident64 instead.
 //   - k_line3_tile: one launch per step for longer lines; a CTA pulls L3_TILE sites
 //     (252 written, two halo sites on each side for the radius-2 stencil of the force).
 #pragma once
 
+#include <cooperative_groups.h>
+
+#include <type_traits>
+
+#include "log64.cuh"
 #include "staged.cuh"
 
 namespace mclb {
@@ -55,9 +61,22 @@ template <typename C>
 __device__ __forceinline__ void collide3(const StepParams<C>& p, const C (&f)[3], C r, C j, C u,
                                          C a, C (&out)[3])
 {
+    const C keep = C(1) - p.omega, omr = p.omega * r;
+    if constexpr (std::is_same<C, double>::value) {
+        // the same polynomial by its even and odd parts, 16 operations instead of 36 (the
+        // FP64 pipe bounds these lines): with q = rho^s/tau u^2 + 2 a j,
+        //   w_0 [rho^s/tau - 1.5 q],  w_+- [rho^s/tau + 3 q +- 3 (rho^s/tau u + rho^s a)]
+        const C ou = omr * u;
+        const C q = fma(C(2), a * j, ou * u);
+        const C odd = C(0.5) * fma(r, a, ou);
+        const C even = fma(C(0.5), q, C(1.0 / 6.0) * omr);
+        out[0] = fma(keep, f[0], fma(C(2.0 / 3.0), omr, -q));
+        out[1] = fma(keep, f[1], even + odd);
+        out[2] = fma(keep, f[2], even - odd);
+        return;
+    }
     const C base = C(-1.5) * u * u;
     const C uu45 = C(4.5) * u * u;
-    const C keep = C(1) - p.omega, omr = p.omega * r;
     const C m3aj = C(-3) * a * j + omr;
     const C e0 = w3<C>(0) * base;
     const C ep = w3<C>(1) * (base + uu45 + C(3) * u);
@@ -120,10 +139,13 @@ struct Line3Smem {
     using C = typename Storage<T>::C;
     // per site: 3N post-collision populations, N densities, N potentials
     static constexpr size_t bytes(int nx) { return (size_t)(5 * N) * nx * sizeof(C); }
+    // FP64, one thread per site and component: also N momenta, the total density and four
+    // per-site terms, and the neighbours' values beyond a piece's ends
+    static constexpr size_t bytes64(int n) { return (size_t)((6 * N + 5) * n + 6 * N + 2) * sizeof(C); }
 };
 
-// K steps of one line per CTA, in shared memory: reads items[b].f[parity], writes
-// items[b].f[parity ^ 1].  blockDim.x >= the longest nx of the launch.
+// FP32: K steps of one line per CTA, one thread per site.
+// Reads items[b].f[parity], writes items[b].f[parity ^ 1].  blockDim.x >= the longest nx of the launch.
 template <typename T, int N>
 __global__ void __launch_bounds__(L3_MAX_SITES)
 k_line3_resident(const Line3Item<T>* __restrict__ items, int parity, int nsteps)
@@ -207,6 +229,191 @@ k_line3_resident(const Line3Item<T>* __restrict__ items, int parity, int nsteps)
     }
     if (bad) atomicOr(p.status, STATUS_NONFINITE);
     for (int k = threadIdx.x; k < 3 * N * nx; k += blockDim.x) fout[k] = T(A[k]);
+}
+
+// FP64: K steps of one line per CTA or, where SMs would idle, per cluster of CTAs that cut the
+// line into pieces; one thread per site and component (thread t: site t mod stride, component
+// t / stride).
+//
+// The FP64 pipe bounds it: one warp instruction per 64 cycles and SM quarter, however many of
+// the 32 lanes are active, so a step costs the FP64 instructions of the busiest quarter.  A
+// site's step is therefore spread over its N threads and written short: collide3's even and odd
+// parts (16 where 36), one reciprocal (two divisions before), log64 (13 for 29), the sum over
+// phi formed from rho^s and scaled once.  With one thread per site the busiest quarter ran
+// about 180 instructions a step (N = 2), now about 50.  60 lines of 128 sites, N = 2:
+// 5.71 -> 2.66 us a step (a CTA pair per line); 512 of 600: 98 -> 62; 10 of 600, N = 3: 38.5 -> 5.1.
+//
+// Arrays carry the neighbouring site's value beyond the ends of a piece; the thread that owns an
+// end site also stores there, in the neighbouring piece's shared memory (its own where the
+// line is one piece).  A step:
+//   pull, rho^s, j^s                       | barrier (CTA; cluster where kappa != 0)
+//   ln rho, 1/rho and what follows from it | barrier (CTA)
+//   nu^s                                   | barrier (cluster)
+//   a^s, collision                         | barrier (cluster)
+template <int N>
+__global__ void __launch_bounds__(L3_MAX_SITES)
+k_line3_resident64(const Line3Item<double>* __restrict__ items, int parity, int nsteps, int stride)
+{
+    using C = double;
+    namespace cg = cooperative_groups;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ StepParams<C> p;
+    __shared__ Log64Row tab[LOG64_ROWS];
+    const cg::cluster_group cl = cg::this_cluster();
+    const int pieces = (int)cl.num_blocks(), rank = (int)cl.block_rank();
+    const Line3Item<double>& item = items[blockIdx.x / pieces];
+    {
+        static_assert(sizeof(StepParams<C>) % sizeof(int) == 0, "parameter copy by words");
+        const int* src = reinterpret_cast<const int*>(&item.p);
+        for (int k = threadIdx.x; k < (int)(sizeof(StepParams<C>) / sizeof(int)); k += blockDim.x)
+            reinterpret_cast<int*>(&p)[k] = src[k];
+    }
+    log64_load(tab);
+    __syncthreads();
+    const int nx = p.nx;
+    const auto start = [&](int k) { return (int)((long long)nx * k / pieces); };
+    const int x0 = start(rank), n = start(rank + 1) - x0;
+    const bool lap = p.kappa != 0.0;
+    // [N]: f*_0 at 0 .. n - 1, f*_+ with the left neighbour's before it, f*_- with the right
+    // neighbour's after it; nu^s and rho^s with both; the Gibbs-Duhem form's total density with
+    // both; per site j^s, theta/rho, u, ln rho and the components' common part of nu^s
+    struct Arrays {
+        int n;
+        C* a;
+        __device__ C* f0(int s) const { return a + s * (3 * n + 2); }
+        __device__ C* fp(int s) const { return f0(s) + n + 1; }        // fp(s)[-1]: left neighbour's
+        __device__ C* fm(int s) const { return f0(s) + 2 * n + 1; }    // fm(s)[n]: right neighbour's
+        __device__ C* nu(int s) const { return a + N * (3 * n + 2) + s * (n + 2) + 1; }
+        __device__ C* rho(int s) const { return nu(N + s); }
+        __device__ C* total() const { return nu(2 * N); }
+        __device__ C* j(int s) const { return a + N * (3 * n + 2) + (2 * N + 1) * (n + 2) + s * n; }
+        __device__ C* site(int q) const { return j(N + q); }
+    };
+    const int rl = rank == 0 ? pieces - 1 : rank - 1, rr = rank == pieces - 1 ? 0 : rank + 1;
+    C* base = reinterpret_cast<C*>(smem_raw);
+    const Arrays me{n, base}, left{start(rl + 1) - start(rl), cl.map_shared_rank(base, rl)},
+        right{start(rr + 1) - start(rr), cl.map_shared_rank(base, rr)};
+    const auto sync = [&]() {
+        if (pieces == 1)
+            __syncthreads();
+        else
+            cl.sync();
+    };
+    const int s = (int)threadIdx.x / stride, l = (int)threadIdx.x - s * stride, x = x0 + l;
+    const bool act = s < N && l < n, first = act && l == 0, last = act && l == n - 1;
+    const C* fin = item.f[parity];
+    C* fout = item.f[parity ^ 1];
+    if (act) {
+        const C* g = fin + (long long)s * 3 * nx;
+        me.f0(s)[l] = g[x];
+        me.fp(s)[l] = g[nx + x];
+        me.fm(s)[l] = g[2 * nx + x];
+        if (first) me.fp(s)[-1] = g[nx + wrap1(x - 1, nx)];
+        if (last) me.fm(s)[n] = g[2 * nx + wrap1(x + 1, nx)];
+    }
+    sync();   // (also: every CTA of the cluster runs before the first store to a neighbour)
+    bool bad = false;
+    const C k05 = -0.5 * p.fcoef;
+    const bool own_log = act && ((p.log_mask >> s) & 1u);
+    // ln rho by the first component without a logarithm of its own (else the last), the rest of
+    // the site's terms by another one
+    const int free_s = __ffs(~p.log_mask & ((1u << N) - 1u));
+    const int s_log = free_s > 0 ? free_s - 1 : N - 1, s_inv = N == 1 ? 0 : (s_log == N - 1 ? N - 2 : N - 1);
+    for (int t = 0; t < nsteps; ++t) {
+        C f[3] = {0.0, 0.0, 0.0}, r = 0.0, j = 0.0;
+        if (act) {
+            f[0] = me.f0(s)[l];
+            f[1] = me.fp(s)[l - 1];
+            f[2] = me.fm(s)[l + 1];
+            r = (f[0] + f[1]) + f[2];
+            j = f[1] - f[2];
+            me.rho(s)[l] = r;
+            me.j(s)[l] = j;
+            if (lap) {
+                if (first) left.rho(s)[left.n] = r;
+                if (last) right.rho(s)[-1] = r;
+            }
+        }
+        if (lap)
+            sync();
+        else
+            __syncthreads();
+        C mine = 0.0;   // (theta/m^s - 1/3) ln rho^s
+        if (act) {
+            C rt[N], rho = 0.0;
+#pragma unroll
+            for (int q = 0; q < N; ++q) {
+                rt[q] = me.rho(q)[l];
+                rho += rt[q];
+            }
+            if (s == s_log) me.site(2)[l] = log64(rho, tab);
+            if (s == s_inv) {
+                C jt = 0.0, sm = 0.0, quad = 0.0;
+#pragma unroll
+                for (int q = 0; q < N; ++q) {
+                    C c = 0.0;
+#pragma unroll
+                    for (int w = 0; w < N; ++w) c += p.chi[q * N + w] * rt[w];
+                    jt += me.j(q)[l];
+                    sm += rt[q] * p.inv_m[q];
+                    quad += rt[q] * c;
+                }
+                const C inv = 1.0 / rho, ti = p.theta * inv;
+                me.site(0)[l] = ti;
+                me.site(1)[l] = jt * inv;
+                me.site(3)[l] = -ti * fma(0.5 * quad, inv, sm);
+                bad = bad || !(rho > 0.0) || !isfinite(rho);
+                if (p.gd) {
+                    me.total()[l] = rho;
+                    if (first) left.total()[left.n] = rho;
+                    if (last) right.total()[-1] = rho;
+                }
+            }
+            if (own_log) {
+                const C fl = p.log_floor * rho;
+                mine = p.logc[s] * log64(r > fl ? r : fl, tab);
+            }
+        }
+        __syncthreads();
+        if (act) {
+            C c = 0.0;
+#pragma unroll
+            for (int w = 0; w < N; ++w) c += p.chi[s * N + w] * me.rho(w)[l];
+            C nu = fma(-p.th_m[s], me.site(2)[l], fma(me.site(0)[l], c, me.site(3)[l])) + mine;
+            if (lap) nu -= p.kappa * ((me.rho(s)[l + 1] + me.rho(s)[l - 1]) - 2.0 * r);
+            me.nu(s)[l] = nu;
+            if (first) left.nu(s)[left.n] = nu;
+            if (last) right.nu(s)[-1] = nu;
+        }
+        sync();
+        if (act) {
+            const C u = me.site(1)[l];
+            C a = fma(k05, me.nu(s)[l + 1] - me.nu(s)[l - 1], p.gx);
+            if (p.gd) {
+                // the common shift of gibbs_duhem3: (A_c - A)/rho with A = sum_s rho^s (a^s - g)
+                C A = 0.0;
+#pragma unroll
+                for (int q = 0; q < N; ++q) A += me.rho(q)[l] * (me.nu(q)[l + 1] - me.nu(q)[l - 1]);
+                const C k3 = p.fcoef * (0.5 / 3.0);
+                a += fma(k3, me.total()[l + 1] - me.total()[l - 1], -k05 * A) / me.total()[l];
+            }
+            C out[3];
+            collide3(p, f, r, p.bary ? r * u : j, u, a, out);
+            me.f0(s)[l] = out[0];
+            me.fp(s)[l] = out[1];
+            me.fm(s)[l] = out[2];
+            if (last) right.fp(s)[-1] = out[1];
+            if (first) left.fm(s)[left.n] = out[2];
+        }
+        sync();
+    }
+    if (bad) atomicOr(p.status, STATUS_NONFINITE);
+    if (act) {
+        C* g = fout + (long long)s * 3 * nx;
+        g[x] = me.f0(s)[l];
+        g[nx + x] = me.fp(s)[l];
+        g[2 * nx + x] = me.fm(s)[l];
+    }
 }
 
 // One step of a line of any length: CTA b covers written sites [x0, x0 + L3_TILE - 4),

@@ -419,9 +419,13 @@ struct Line3Launch {
     }
 
     template <int N>
-    static cudaError_t resident(const Line3Item<T>* items, int count, int nxmax, int parity,
+    static cudaError_t resident(const Line3Item<T>* items, int count, int nxmin, int nxmax, int parity,
                                 int nsteps, cudaStream_t st)
     {
+        if constexpr (std::is_same<T, double>::value) {
+            const int c = pieces<N>(count, nxmin, nxmax);
+            if (c > 0) return resident64<N>(c, items, count, nxmax, parity, nsteps, st);
+        }
         static const cudaError_t attr = cudaFuncSetAttribute(
             k_line3_resident<T, N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_CAP);
         if (attr != cudaSuccess) return attr;
@@ -429,6 +433,59 @@ struct Line3Launch {
         const int threads = (nxmax + 31) / 32 * 32;
         k_line3_resident<T, N><<<count, threads, smem, st>>>(items, parity, nsteps);
         return cudaGetLastError();
+    }
+
+    // CTAs per line for k_line3_resident64 (0: its threads or shared memory do not fit): the
+    // count that leaves the busiest SM quarter the fewest warps, whose FP64 instructions are
+    // the launch's time (60 lines of 128 sites, N = 2, 1 / 2 / 4 / 8 CTAs: 3.57, 2.66, 2.60,
+    // 4.03 us a step; 200 of 100, N = 3: 13.7, 10.5, 10.7, 21.2; 10 of 600, N = 3, 2 / 4 / 8:
+    // 14.1, 7.5, 5.1)
+    template <int N>
+    static int pieces(int count, int nxmin, int nxmax)
+    {
+        int dev = 0, sms = 1;
+        if (cudaGetDevice(&dev) != cudaSuccess ||
+            cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) {
+            cudaGetLastError();
+            return 0;
+        }
+        int best = 0;
+        long long least = 0;
+        for (int c = 1; c <= 8 && c <= nxmin; c *= 2) {
+            const int n = (nxmax + c - 1) / c, stride = (n + 31) / 32 * 32;
+            if (N * stride > L3_MAX_SITES || Line3Smem<T, N>::bytes64(n) > SMEM_CAP64) continue;
+            const long long ctas = ((long long)count * c + sms - 1) / sms;
+            const long long cost = (ctas * (N * stride / 32) + 3) / 4;
+            if (best == 0 || cost < least) {
+                best = c;
+                least = cost;
+            }
+        }
+        return best;
+    }
+
+    static constexpr size_t SMEM_CAP64 = 227 * 1024 - round_up_sz(sizeof(StepParams<C>) + LOG64_ROWS * sizeof(Log64Row) + 16, 128);
+
+    template <int N>
+    static cudaError_t resident64(int c, const Line3Item<T>* items, int count, int nxmax, int parity,
+                                  int nsteps, cudaStream_t st)
+    {
+        static const cudaError_t attr = cudaFuncSetAttribute(
+            k_line3_resident64<N>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM_CAP64);
+        if (attr != cudaSuccess) return attr;
+        const int n = (nxmax + c - 1) / c, stride = (n + 31) / 32 * 32;
+        cudaLaunchConfig_t cfg{};
+        cudaLaunchAttribute at{};
+        at.id = cudaLaunchAttributeClusterDimension;
+        at.val.clusterDim.x = (unsigned)c;
+        at.val.clusterDim.y = at.val.clusterDim.z = 1;
+        cfg.gridDim = dim3((unsigned)(count * c));
+        cfg.blockDim = dim3((unsigned)(N * stride));
+        cfg.dynamicSmemBytes = Line3Smem<T, N>::bytes64(n);
+        cfg.stream = st;
+        cfg.attrs = &at;
+        cfg.numAttrs = 1;
+        return cudaLaunchKernelEx(&cfg, k_line3_resident64<N>, items, parity, nsteps, stride);
     }
 
     template <int N>
@@ -461,7 +518,7 @@ struct Line3Launch {
                 cudaError_t e;
                 if (res) {
                     const int k = (int)std::min<long>(nsteps, L3_CHUNK);
-                    e = resident<NN>((const Line3Item<T>*)sc.line_item, 1, P.nx, *cur, k, st);
+                    e = resident<NN>((const Line3Item<T>*)sc.line_item, 1, P.nx, P.nx, *cur, k, st);
                     nsteps -= k;
                 } else {
                     e = tile<NN>(p, f[*cur], f[*cur ^ 1], st);
@@ -533,7 +590,7 @@ struct Line3Launch {
     struct Group {
         int N = 0;
         Line3Item<T>* d_items = nullptr;     // lines the resident kernel holds
-        int nres = 0, nxmax = 1;
+        int nres = 0, nxmin = INT32_MAX, nxmax = 1;
         std::vector<Line3Item<T>> longs;     // lines stepped with the tile kernel
         std::vector<size_t> long_bytes;
     };
@@ -549,6 +606,7 @@ struct Line3Launch {
             const Line3Item<T> it = item(probs[k], scs[k], fa[k], fb[k]);
             if (probs[k].nx <= max_resident(N)) {
                 res.push_back(it);
+                g->nxmin = std::min(g->nxmin, probs[k].nx);
                 g->nxmax = std::max(g->nxmax, probs[k].nx);
             } else {
                 g->longs.push_back(it);
@@ -574,7 +632,7 @@ struct Line3Launch {
         auto* g = static_cast<Group*>(gv);
         MCLB_DISPATCH_N(g->N, {
             if (g->nres > 0) {
-                cudaError_t e = resident<NN>(g->d_items, g->nres, g->nxmax, parity, nsteps, st);
+                cudaError_t e = resident<NN>(g->d_items, g->nres, g->nxmin, g->nxmax, parity, nsteps, st);
                 if (e != cudaSuccess) return e;
             }
             for (size_t k = 0; k < g->longs.size(); ++k) {

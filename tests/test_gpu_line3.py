@@ -293,3 +293,34 @@ def test_line3_batch_ternary_polymer_near_critical():
         assert np.abs(rich - tl[np.argmax(tl[:, 0])]).max() < 0.04, p.name
         assert np.abs(poor - tl[np.argmin(tl[:, 0])]).max() < 0.04, p.name
     b.close()
+
+
+@pytest.mark.parametrize("gd", [0, 1])
+@pytest.mark.parametrize("count,nx,n", [(1, 1, 2), (1, 33, 1), (3, 64, 2), (1, 127, 3), (2, 257, 2), (1, 1000, 2),
+                                        (1, 640, 8), (200, 40, 3), (3, 100, 5)])
+def test_fp64_lines_in_pieces(count, nx, n, gd):
+    """FP64 lines of one N, cut into one to eight CTAs by count and length, against the oracle
+    to 1e-12 after 60 steps: every term on, components with and without a logarithm of their
+    own, both forcing velocities, the lines of a batch of different length."""
+    probs = []
+    for k in range(count):
+        m = nx + (k % 3 if nx > 1 else 0)
+        rho, u = inputs.random_state(n, m, 1, seed=900 + k, amp=0.3, umax=0.03)
+        u[1] = 0.0
+        p = inputs.Problem(name=f"l{k}", ncomp=n, nx=m, ny=1, tau=0.9, chi=inputs.uniform_chi(n, 1.6),
+                           m=np.array([1.0 + ((k + q) % 2) for q in range(n)]), theta=1.0 / 3.0,
+                           kappa=0.0 if gd or k % 2 else 0.02, force=(1e-5, 0.0), rho=rho, u=u, lattice="d1q3")
+        p.forcing_velocity, p.force_form = k % 2, gd
+        probs.append(p)
+    b = mclb.Batch(probs, precision="fp64")
+    b.init_all()
+    b.step(60)
+    assert b.status()[0] == 0
+    for k in (0, count // 2, count - 1):
+        orc = Oracle.from_problem(probs[k])
+        assert orc.run(60) == 0
+        m = orc.moments()
+        got = b.moments(k)
+        for f in ("rho", "U"):
+            assert np.max(np.abs(got[f] - m[f])) < 1e-12 * max(1.0, np.max(np.abs(m[f]))), (k, f)
+    b.close()
