@@ -122,6 +122,7 @@ struct StepParams {
     C logc[NMAX];         // theta / m^s - 1/3: coefficient of ln rho^s in nu^s
     C m_inv_m1[NMAX];     // 1/m^s - 1
     C inv_m[NMAX];        // 1/m^s
+    C dm[NMAX];           // 1/m^s - 1/m^0: sum_s phi^s/m^s less the constant 1/m^0 (sum_s phi^s = 1)
     C m[NMAX];
     unsigned int log_mask; // bit s set when logc[s] != 0
     int withhold;          // test hook: the single-pass kernel issues no copies
@@ -161,6 +162,7 @@ inline StepParams<C> make_params(const Problem& P, unsigned int* status)
         if (c != 0.0) p.log_mask |= 1u << a;
         p.m_inv_m1[a] = C(1.0 / P.m[a] - 1.0);
         p.inv_m[a] = C(1.0 / P.m[a]);
+        p.dm[a] = C(1.0 / P.m[a] - 1.0 / P.m[0]);
         p.m[a] = C(P.m[a]);
     }
     p.withhold = P.withhold;

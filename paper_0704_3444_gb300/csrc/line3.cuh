@@ -238,8 +238,8 @@ k_line3_resident(const Line3Item<T>* __restrict__ items, int parity, int nsteps)
 // The FP64 pipe bounds it: one warp instruction per 64 cycles and SM quarter, however many of
 // the 32 lanes are active, so a step costs the FP64 instructions of the busiest quarter.  A
 // site's step is therefore spread over its N threads and written short: collide3's even and odd
-// parts (16 where 36), one reciprocal (two divisions before), log64 (13 for 29), the sum over
-// phi formed from rho^s and scaled once.  With one thread per site the busiest quarter ran
+// parts (16 where 36), one reciprocal (two divisions before), log64 (13 for 29), the sums over
+// phi formed from rho^s and scaled once, without the constants of nu^s, which have no gradient.  With one thread per site the busiest quarter ran
 // about 180 instructions a step (N = 2), now about 50.  60 lines of 128 sites, N = 2:
 // 5.71 -> 2.66 us a step (a CTA pair per line); 512 of 600: 98 -> 62; 10 of 600, N = 3: 38.5 -> 5.1.
 //
@@ -355,7 +355,7 @@ k_line3_resident64(const Line3Item<double>* __restrict__ items, int parity, int 
 #pragma unroll
                     for (int w = 0; w < N; ++w) c += p.chi[q * N + w] * rt[w];
                     jt += me.j(q)[l];
-                    sm += rt[q] * p.inv_m[q];
+                    sm += rt[q] * p.dm[q];
                     quad += rt[q] * c;
                 }
                 const C inv = 1.0 / rho, ti = p.theta * inv;

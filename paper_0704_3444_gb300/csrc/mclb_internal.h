@@ -87,6 +87,7 @@ struct FusedPlan {
 // (rows.cuh, lx = 0).
 struct TilePlan {
     int lx, ty;
+    int parts;
     int gx, gy;
     int threads;
     size_t smem;

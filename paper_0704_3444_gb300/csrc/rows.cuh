@@ -151,21 +151,20 @@ k_rows(const float* __restrict__ fin, float* __restrict__ fout, const __grid_con
         const int yy = y0 - 1 + t;
         // rows beyond a wall are the mirror images of those next to it
         const int up = (WALLS && yy <= 0) ? 0 : -32, dn = (WALLS && yy >= p.ny - 1) ? 0 : 32;
-        float rr[N], lap[N], nu[N];
+        float rr[N], nu[N], rho, inv;
+#pragma unroll
+        for (int q = 0; q < N; ++q) rr[q] = R[q][t + 1][lane];
+        tile_nu<float, N>(p, rr, nullptr, 0, 1, nu, rho, inv);
 #pragma unroll
         for (int q = 0; q < N; ++q) {
             const float* g = &R[q][t + 1][lane];
-            rr[q] = g[0];
-            lap[q] = 0.0f;
             if (p.kappa != 0.0f) {
                 const float ax = (g[-1] + g[1]) + (g[up] + g[dn]);
                 const float di = (g[up - 1] + g[up + 1]) + (g[dn - 1] + g[dn + 1]);
-                lap[q] = fmaf(2.0f / 3.0f, ax, fmaf(1.0f / 6.0f, di, (-10.0f / 3.0f) * rr[q]));
+                nu[q] = fmaf(-p.kappa, fmaf(2.0f / 3.0f, ax, fmaf(1.0f / 6.0f, di, (-10.0f / 3.0f) * rr[q])), nu[q]);
             }
+            NU[q][t][lane] = nu[q];
         }
-        site_nu<float, N>(p, rr, lap, nu);
-#pragma unroll
-        for (int q = 0; q < N; ++q) NU[q][t][lane] = nu[q];
     }
     // ---- u of the tile rows, from the last warp down (the first have the potentials)
     for (int l = ROWS_WPC * N - 1 - warp; l < ROWS_Y; l += ROWS_WPC * N) {

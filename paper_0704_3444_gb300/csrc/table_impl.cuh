@@ -312,20 +312,20 @@ struct TileLaunch {
     // Most sites x components for which a tile kernel beats the march (measured on both sides of
     // each line, us per step, tile / march; between walls the march also pays three band
     // launches, about 20 us):
-    //   FP64: it runs at the FP64 pipe's rate on every SM, and collide_poly needs fewer FP64
-    //     operations: 64 x 64 x 2 10.8 / 107, 1024^2 x 2 652 / 745, 2048^2 x 2 2589 / 2609; five
-    //     and more components 300 x 200 x 5 116 / 206, 1024^2 x 5 1819 / 1493
+    //   FP64: it runs at the FP64 pipe's rate on every SM with fewer FP64 instructions a site:
+    //     64 x 64 x 2 9.73 / 107, 2048^2 x 2 2323 / 2613, 2048^2 x 3 3474 / 3802, 600^2 x 6 758 /
+    //     1233, 500^2 x 8 714 / 1130, Gibbs-Duhem 1024^2 x 3 967 / 1132: every size, but
+    //     1024^2 x 4 1270 / 1230, 1024^2 x 5 1640 / 1494
     //   FP32 (k_rows): 1000^2 x 1 18.1 / 26.3; 700^2 x 2 20.5 / 22.3, 1024^2 x 2 38 / 37;
     //     512 x 384 x 3 14.7 / 18.5, 700 x 600 x 3 29.8 / 25.7; 400^2 x 4 21.7 / 20.1;
     //     300^2 x 5 13.5 / 19.4, 500 x 450 x 5 24.9 / 23.6; walls 1000 x 333 x 3 21 / 39,
     //     1500 x 1200 x 3 107 / 95.  k_tile, six and more: 300^2 x 6 20.0 / 23.1
     //   16-bit: 400 x 300 x 4 19.7 / 22.8, 400^2 x 5 33 / 30; walls 1000 x 700 x 3 65.5 / 66.6
-    //   Gibbs-Duhem: FP64 1024^2 x 3 1098 / 1131; FP32 300^2 x 2 10.4 / 16.0, 512 x 384 x 3
-    //     22.8 / 18.5
+    //   FP32 Gibbs-Duhem: 300^2 x 2 10.3 / 15.8, 512 x 384 x 3 22.8 / 18.5
     static long long most(const Problem& P)
     {
         const int N = P.N;
-        if (sizeof(C) == 8) return N >= 5 ? 1500000 : (P.force_form == FORCE_GIBBS_DUHEM ? 3000000 : 8000000);
+        if (sizeof(C) == 8) return N == 4 || N == 5 ? 3000000 : 1LL << 40;
         if (P.force_form == FORCE_GIBBS_DUHEM) return 350000;
         if (Storage<T>::shifted) return P.walls ? 2000000 : 600000;
         if (P.walls) return 4000000;
@@ -360,8 +360,13 @@ struct TileLaunch {
         pl.gx = (P.nx + (1 << pl.lx) - 1) >> pl.lx;
         pl.gy = (P.ny + ty - 1) / ty;
         pl.threads = P.N * (ty << pl.lx);
+        pl.parts = 1;
+        if (sizeof(C) == 8 && small && P.N <= 4) {   // a CTA of few warps: twice the threads
+            pl.threads *= 2;
+            pl.parts = std::min(P.N, 2);
+        }
         pl.smem = sizeof(C) * tile_smem_values(P.N, 1 << pl.lx, ty, gd);
-        pl.ok = pl.threads <= tile_max_threads<T>() && pl.smem <= 48 * 1024 && pl.gy < 65536 &&
+        pl.ok = pl.threads <= tile_max_threads<T>() && pl.smem <= 44 * 1024 && pl.gy < 65536 &&
                 (long long)P.plane * P.N < (1LL << 31);
         return pl;
     }
@@ -386,7 +391,7 @@ struct TileLaunch {
         }
         MCLB_DISPATCH_N(P.N, {
             return launch_dependent(k_tile<T, NN>, dim3(pl.gx, pl.gy), pl.threads, pl.smem, st,
-                                    (const T*)fin, (T*)fout, rs, p, pl.lx, pl.ty);
+                                    (const T*)fin, (T*)fout, rs, p, pl.lx, pl.ty, pl.parts);
         });
     }
 };

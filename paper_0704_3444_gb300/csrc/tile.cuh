@@ -18,17 +18,19 @@
 
 #include <type_traits>
 
+#include "log64.cuh"
 #include "tma.cuh"
 
 namespace mclb {
 
-// Threads per CTA and registers per thread at most: 56 and 80 registers keep two to three CTAs
+// Threads per CTA and registers per thread at most: 56 registers, and 80 in FP64
+// up to four components, keep two to three CTAs
 // of 16 x 8 sites on an SM (uncapped the compiler takes 72 and 128: 1000 x 333 x 3 FP32
 // 31.6 -> 26.9 us, 512 x 512 x 2 FP64 188 -> 171 us).
 template <typename T>
 constexpr int tile_max_threads() { return sizeof(typename Storage<T>::C) == 8 ? 512 : 768; }
 template <typename T>
-constexpr int tile_max_regs() { return sizeof(typename Storage<T>::C) == 8 ? 80 : 56; }
+constexpr int tile_max_regs(int n) { return sizeof(typename Storage<T>::C) == 8 ? (n <= 4 ? 80 : 128) : 56; }
 
 // Programmatic dependent launch: wait until the kernels this one depends on are complete and
 // their writes visible; let the next kernel of the stream be scheduled (its own wait still
@@ -104,8 +106,9 @@ __device__ __forceinline__ C sum9(const C (&v)[Q])
 //   f*_i = (1 - 1/tau) f_i + w_i [rho^s/tau - (Cxx + Cyy)/3 + L.v + C:vv],
 // whose parts even and odd in v serve two opposite velocities at once: 57 operations where
 // the direction-by-direction form takes 45 plus 36 for the site's e_i, which here every
-// component's thread would form again.  The constant w_i rho^s/tau enters last (see
-// eq_weights on why it is not rounded together with the velocity terms).
+// component's thread would form again.  The constant w_i rho^s/tau enters last (see eq_weights
+// on why it is not rounded together with the velocity terms; summed with them first, 9
+// operations fewer, the error of U on 64 x 64 FP64 grew from 2.2e-15 to 3.3e-15).
 template <typename C>
 __device__ __forceinline__ void collide_poly(const StepParams<C>& p, const C (&f)[Q], C r, C jx, C jy,
                                              C ux, C uy, C ax, C ay, C shift, C (&out)[Q])
@@ -133,6 +136,45 @@ __device__ __forceinline__ void collide_poly(const StepParams<C>& p, const C (&f
     put(6, em - om);
 }
 
+__device__ __forceinline__ float tile_log(float x, const Log64Row*) { return dev_log(x); }
+__device__ __forceinline__ double tile_log(double x, const Log64Row* tab) { return log64(x, tab); }
+
+// nu^s without its gradient term, as in site_nu with the sums over phi formed from rho^s and
+// scaled once, of the components that `part` of `parts` takes; also rho and 1/rho.  Constants
+// have no gradient and are left out (theta (1/m^s - 1), and theta/m^0 of theta sum phi^s/m^s: what
+// is left of that sum vanishes for equal m), which also leaves less to round.
+template <typename C, int N>
+__device__ __forceinline__ void tile_nu(const StepParams<C>& p, const C (&r)[N], const Log64Row* tab, int part,
+                                        int parts, C (&nu)[N], C& rho, C& inv)
+{
+    rho = r[0];
+#pragma unroll
+    for (int s = 1; s < N; ++s) rho += r[s];
+    inv = C(1) / rho;
+    C acc[N], sm = C(0), quad = C(0);
+#pragma unroll
+    for (int s = 0; s < N; ++s) {
+        C a = C(0);
+#pragma unroll
+        for (int t = 0; t < N; ++t) a += p.chi[s * N + t] * r[t];
+        acc[s] = a;
+        sm += r[s] * p.dm[s];
+        quad += r[s] * a;
+    }
+    const C ti = p.theta * inv;
+    const C G = -ti * fma(C(0.5) * quad, inv, sm);
+    const C lnr = tile_log(rho, tab);
+#pragma unroll
+    for (int s = 0; s < N; ++s) {
+        if (parts > 1 && s % parts != part) continue;
+        nu[s] = fma(-p.th_m[s], lnr, fma(ti, acc[s], G));
+        if ((p.log_mask >> s) & 1u) {
+            const C fl = p.log_floor * rho;
+            nu[s] += p.logc[s] * tile_log(r[s] > fl ? r[s] : fl, tab);
+        }
+    }
+}
+
 // rho^s of every site and component (one per thread), for k_tile's rs.
 template <typename T>
 __global__ void __launch_bounds__(128)
@@ -152,14 +194,19 @@ k_tile_rho(const T* __restrict__ f, typename Storage<T>::C* __restrict__ rs,
 }
 
 // One timestep fin -> fout on the tiles blockIdx: columns [TX bx, ...), rows [y0, y0 + TY) with
-// y0 = TY by, TX = 1 << lx.  blockDim.x = N TX TY.  rs: the rho^s field of fin, read around the
-// tile instead of pulling there, or null.
+// y0 = TY by, TX = 1 << lx.  blockDim.x = N TX TY, or more: threads beyond those pull around the
+// tile while the others pull the tile, and parts > 1 spreads a site's potentials over as many
+// threads -- for tiles of so few warps that SM quarters would idle.  rs: the rho^s field of
+// fin, read around the tile instead of pulling there, or null.
 template <typename T, int N>
-__global__ void __launch_bounds__(tile_max_threads<T>()) __maxnreg__(tile_max_regs<T>())
+__global__ void __launch_bounds__(tile_max_threads<T>()) __maxnreg__(tile_max_regs<T>(N))
 k_tile(const T* __restrict__ fin, T* __restrict__ fout, const typename Storage<T>::C* __restrict__ rs,
-       const __grid_constant__ StepParams<typename Storage<T>::C> p, int lx, int ty)
+       const __grid_constant__ StepParams<typename Storage<T>::C> p, int lx, int ty, int parts64)
 {
     using C = typename Storage<T>::C;
+    constexpr bool F64 = sizeof(C) == 8;
+    const int parts = F64 ? parts64 : 1;
+    __shared__ Log64Row tab[F64 ? LOG64_ROWS : 1];
     extern __shared__ __align__(16) unsigned char tile_raw[];
     const int TX = 1 << lx, SITES = ty << lx;
     const int EX = TX + 4, EY = ty + 4, NX = TX + 2, NY = ty + 2;
@@ -173,6 +220,7 @@ k_tile(const T* __restrict__ fin, T* __restrict__ fout, const typename Storage<T
 
     const int tid = threadIdx.x;
     const int s = tid / SITES, site = tid - s * SITES;
+    const bool mine = !F64 || s < N;   // (else a thread beyond the tile's)
     const int tx = site & (TX - 1), tyy = site >> lx;
     const int x0 = blockIdx.x << lx, y0 = blockIdx.y * ty;
     const int x = x0 + tx, y = y0 + tyy;
@@ -180,14 +228,16 @@ k_tile(const T* __restrict__ fin, T* __restrict__ fout, const typename Storage<T
     // (lanes beyond the lattice compute some site's values and store nothing)
     const int xlast = p.nx + 1;
 
+    if constexpr (F64) log64_load(tab);
     // the previous step's populations are complete from here on
     grid_dependency_wait();
 
     // ---- rho^s on the tile and two around it; j^s on the tile
-    C f[Q];
-    tile_pull<T, C>(fin, p, s, min(x, xlast), wrap_any(y, p.ny), f);
+    C f[Q], r = C(0), jx = C(0), jy = C(0);
+    if (mine) tile_pull<T, C>(fin, p, s, min(x, xlast), wrap_any(y, p.ny), f);
     const int ring2 = EX * EY - SITES;
-    for (int k = site; k < ring2; k += SITES) {
+    // item k of the surroundings of component c
+    auto around = [&](int c, int k) {
         int q = k, ex, ey;
         if (q < 4 * EX) {                      // the two rows above, then the two below
             ey = q / EX;
@@ -201,29 +251,38 @@ k_tile(const T* __restrict__ fin, T* __restrict__ fout, const typename Storage<T
         const int yr = wrap_any(y0 - 2 + ey, p.ny);
         C rv;
         if (rs) {
-            rv = rs[s * p.S + yr * p.nx + wrap_any(x0 - 2 + ex, p.nx)];
+            rv = rs[c * p.S + yr * p.nx + wrap_any(x0 - 2 + ex, p.nx)];
         } else {
             C v[Q];
-            tile_pull<T, C>(fin, p, s, min(x0 - 2 + ex, xlast), yr, v);
+            tile_pull<T, C>(fin, p, c, min(x0 - 2 + ex, xlast), yr, v);
             rv = sum9(v);
         }
-        R[(s * EY + ey) * EX + ex] = rv;
+        R[(c * EY + ey) * EX + ex] = rv;
+    };
+    const int extra = F64 ? (int)blockDim.x - N * SITES : 0;
+    if (extra > 0) {
+        for (int k = tid - N * SITES; k >= 0 && k < N * ring2; k += extra) around(k / ring2, k % ring2);
+    } else {
+        for (int k = site; k < ring2; k += SITES) around(s, k);
     }
-    const C r = sum9(f);
-    C jx, jy;
-    {
+    if (mine) {
+        r = sum9(f);
         const C a = f[5] - f[7], b = f[6] - f[8];
         jx = (f[1] - f[3]) + (a - b);
         jy = (f[2] - f[4]) + (a + b);
+        R[(s * EY + tyy + 2) * EX + tx + 2] = r;
+        J[s * SITES + site] = jx;
+        J[(N + s) * SITES + site] = jy;
     }
-    R[(s * EY + tyy + 2) * EX + tx + 2] = r;
-    J[s * SITES + site] = jx;
-    J[(N + s) * SITES + site] = jy;
     __syncthreads();
     grid_dependents_launch();
 
     // ---- nu^s on the tile and one around it; u on the tile
-    for (int k = tid; k < NX * NY; k += N * SITES) {
+    const int npad = (NX * NY + 31) / 32 * 32;   // (a warp's threads take the same part)
+    const int threads = F64 ? (int)blockDim.x : N * SITES;
+    for (int it = tid; it < (F64 ? npad * parts : NX * NY); it += threads) {
+        const int part = F64 ? it / npad : 0, k = it - part * npad;
+        if (F64 && k >= NX * NY) continue;
         int bx, by;
         if (k < SITES) {
             bx = (k & (TX - 1)) + 1;
@@ -243,27 +302,24 @@ k_tile(const T* __restrict__ fin, T* __restrict__ fout, const typename Storage<T
         const C* c = R + (by + 1) * EX + bx + 1;
         // rows beyond a wall are the mirror images of those next to it
         const int up = (p.walls && yy <= 0) ? 0 : -EX, dn = (p.walls && yy >= p.ny - 1) ? 0 : EX;
-        C rr[N], lap[N], nu[N];
+        C rr[N], nu[N], rho, inv;
+#pragma unroll
+        for (int t = 0; t < N; ++t) rr[t] = c[t * EX * EY];
+        tile_nu<C, N>(p, rr, tab, part, parts, nu, rho, inv);
 #pragma unroll
         for (int t = 0; t < N; ++t) {
+            if (parts > 1 && t % parts != part) continue;
             const C* g = c + t * EX * EY;
-            rr[t] = g[0];
-            lap[t] = C(0);
             if (p.kappa != C(0)) {
                 const C ax = (g[-1] + g[1]) + (g[up] + g[dn]);
                 const C di = (g[up - 1] + g[up + 1]) + (g[dn - 1] + g[dn + 1]);
-                lap[t] = fma(C(2.0 / 3.0), ax, fma(C(1.0 / 6.0), di, C(-10.0 / 3.0) * rr[t]));
+                nu[t] = fma(-p.kappa, fma(C(2.0 / 3.0), ax, fma(C(1.0 / 6.0), di, C(-10.0 / 3.0) * rr[t])), nu[t]);
             }
+            NU[(t * NY + by) * NX + bx] = nu[t];
         }
-        site_nu<C, N>(p, rr, lap, nu);
-#pragma unroll
-        for (int t = 0; t < N; ++t) NU[(t * NY + by) * NX + bx] = nu[t];
-        C rho = C(0);
-#pragma unroll
-        for (int t = 0; t < N; ++t) rho += rr[t];
+        if (part != parts - 1) continue;
         if (p.gd) RT[by * NX + bx] = rho;
         if (k < SITES) {
-            const C inv = C(1) / rho;
             C ux = C(0), uy = C(0);
 #pragma unroll
             for (int t = 0; t < N; ++t) {
@@ -286,15 +342,20 @@ k_tile(const T* __restrict__ fin, T* __restrict__ fout, const typename Storage<T
         gx = fma(C(1.0 / 3.0), g[1] - g[-1], C(1.0 / 12.0) * ((ne - nw) + (se - sw)));
         gy = fma(C(1.0 / 3.0), g[dn] - g[up], C(1.0 / 12.0) * ((ne - se) + (nw - sw)));
     };
-    C ax, ay;
-    grad(NU + (s * NY + tyy + 1) * NX + tx + 1, ax, ay);
-    ax = fma(-p.fcoef, ax, p.gx);
-    ay = fma(-p.fcoef, ay, p.gy);
+    C ax = C(0), ay = C(0);
+    if (mine) {
+        grad(NU + (s * NY + tyy + 1) * NX + tx + 1, ax, ay);
+        ax = fma(-p.fcoef, ax, p.gx);
+        ay = fma(-p.fcoef, ay, p.gy);
+    }
     if (p.gd) {
         // the common shift (A_c - A)/rho of every component (gibbs_duhem_shift)
-        A[s * SITES + site] = ax - p.gx;
-        A[(N + s) * SITES + site] = ay - p.gy;
+        if (mine) {
+            A[s * SITES + site] = ax - p.gx;
+            A[(N + s) * SITES + site] = ay - p.gy;
+        }
         __syncthreads();
+        if (!mine) return;
         C sx = C(0), sy = C(0), grx, gry;
 #pragma unroll
         for (int t = 0; t < N; ++t) {
@@ -307,7 +368,7 @@ k_tile(const T* __restrict__ fin, T* __restrict__ fout, const typename Storage<T
         ax += (k * grx - sx) * it;
         ay += (k * gry - sy) * it;
     }
-    if (!own) return;
+    if (!mine || !own) return;
     const C ux = U[site], uy = U[SITES + site];
     C fjx, fjy, out[Q];
     forcing_momentum(p, r, jx, jy, ux, uy, fjx, fjy);
