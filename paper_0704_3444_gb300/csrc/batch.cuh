@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "march.cuh"
+#include "rows.cuh"
 #include "staged.cuh"
 
 namespace mclb {
@@ -66,6 +67,7 @@ struct alignas(64) MarchItem {
     CUtensorMap maps2[2][4];
     StepParams<typename Storage<T>::C> p;
     T* f[2];
+    typename Storage<T>::C* rs;   // density scratch (N * S)
 };
 
 // One CTA of the batched march: instance, first written column, first row, rows.
@@ -100,6 +102,62 @@ kb_march(const MarchItem<T>* __restrict__ items, const MarchCta* __restrict__ ct
     __syncthreads();
     march_cta<T, N, G>(&maps[parity][0], &maps[parity][1], &maps[parity ^ 1][2], &maps[parity ^ 1][3],
                        it.f[parity ^ 1], ps, c.x0, c.y0, c.H, smem);
+}
+
+// A CTA's instance parameters into shared memory (ends with a barrier).
+template <typename P>
+__device__ __forceinline__ void copy_params(P& dst, const P& src)
+{
+    static_assert(sizeof(P) % sizeof(int) == 0, "parameter copy by words");
+    for (int k = threadIdx.x; k < (int)(sizeof(P) / sizeof(int)); k += blockDim.x)
+        reinterpret_cast<int*>(&dst)[k] = reinterpret_cast<const int*>(&src)[k];
+    __syncthreads();
+}
+
+// The tile schedules over the instances of a group; ctas[]: instance, first column, first row,
+// rows.  FP32: the row tiles of rows.cuh, down the CTA's rows.
+template <int N>
+__global__ void __launch_bounds__(32 * ROWS_WPC * N, rows_ctas(N))
+kb_rows(const MarchItem<float>* __restrict__ items, const MarchCta* __restrict__ ctas, int parity)
+{
+    __shared__ StepParams<float> ps;
+    const MarchCta c = ctas[blockIdx.x];
+    const MarchItem<float>& it = items[c.inst];
+    copy_params(ps, it.p);
+    const float* fin = it.f[parity];
+    float* fout = it.f[parity ^ 1];
+    for (int y = c.y0; y < c.y0 + c.H; y += ROWS_Y) rows_tile<N, false>(fin, fout, ps, c.x0, y);
+}
+
+// FP64: rho^s of every site, then the tiles of tile.cuh with those around each tile read back.
+template <int N>
+__global__ void __launch_bounds__(tile_max_threads<double>())
+kb_tile_rho(const MarchItem<double>* __restrict__ items, const MarchCta* __restrict__ ctas, int parity, int lx,
+            int ty)
+{
+    __shared__ StepParams<double> ps;
+    const MarchCta c = ctas[blockIdx.x];
+    const MarchItem<double>& it = items[c.inst];
+    copy_params(ps, it.p);
+    const int sites = ty << lx;
+    for (int k = threadIdx.x; k < N * sites; k += blockDim.x) {
+        const int s = k / sites, q = k - s * sites;
+        const int x = c.x0 + (q & ((1 << lx) - 1)), y = c.y0 + (q >> lx);
+        if (x >= ps.nx || y >= ps.ny) continue;
+        double v[Q];
+        tile_pull<double, double>(it.f[parity], ps, s, x, y, v);
+        it.rs[s * ps.S + (long long)y * ps.nx + x] = sum9(v);
+    }
+}
+template <int N>
+__global__ void __launch_bounds__(tile_max_threads<double>()) __maxnreg__(tile_max_regs<double>(N))
+kb_tile(const MarchItem<double>* __restrict__ items, const MarchCta* __restrict__ ctas, int parity, int lx, int ty)
+{
+    __shared__ StepParams<double> ps;
+    const MarchCta c = ctas[blockIdx.x];
+    const MarchItem<double>& it = items[c.inst];
+    copy_params(ps, it.p);
+    tile_step<double, N>(it.f[parity], it.f[parity ^ 1], it.rs, ps, c.x0, c.y0, lx, ty, 1);
 }
 
 // Ghost columns of every instance's new buffer (parity ^ 1), laid out per instance as in
@@ -151,6 +209,11 @@ struct BatchGroup {
     std::vector<int> cand_waves;
     std::vector<int> cand_geo;   // 0: MarchGeom (wide strips), 1: MarchNarrow
     int pick = 0;
+    // the tile schedules, in place of the march where use_tiles
+    bool use_tiles = false;
+    MarchCta* tiles = nullptr;
+    int ntiles = 0;
+    int lx = 0, ty = 0;          // FP64 tile shape
     long long* gstart = nullptr;
     int* gfirst = nullptr;      // first ghost block of each instance
     int* gblk2inst = nullptr;   // instance of each ghost block
@@ -177,6 +240,56 @@ std::vector<MarchCta> march_ctas(int count, const Problem* probs, int slots, int
     }
     std::stable_sort(v.begin(), v.end(), [](const MarchCta& a, const MarchCta& b) { return a.H > b.H; });
     return v;
+}
+
+// Whether a group's instances step by tiles instead of the march.
+//   FP32: row tiles where every instance has rows enough and the group keeps the GPU busy (48
+//     instances of 32^2 to 512^2, N = 2 and 3: 153 us a step, 184 by the march with its ghost
+//     launch; 300 of 32^2 to 200^2: 231 / 307), up to the five components whose CTAs share an SM.
+//   FP64: the tiles spend fewer FP64 instructions than the march (table_impl.cuh has both sides),
+//     but for four and five components.
+template <typename T>
+bool batch_takes_tiles(int N, int count, const Problem* probs)
+{
+    long long work = 0;
+    int rows = INT32_MAX;
+    for (int k = 0; k < count; ++k) {
+        work += probs[k].S * N;
+        rows = std::min(rows, probs[k].ny);
+        if ((long long)probs[k].plane * N >= (1LL << 31)) return false;
+    }
+    if (std::is_same<T, float>::value) return N <= ROWS_NMAX && rows >= ROWS_MIN_NY && work >= 1000000;
+    if (std::is_same<T, double>::value) return N != 4 && N != 5;
+    return false;
+}
+
+// Tables of the tile schedules: FP32 row tiles two deep (a CTA copies its parameters once for both).
+constexpr int BATCH_TILE_ROWS = 2 * ROWS_Y;
+inline std::vector<MarchCta> tile_ctas(int count, const Problem* probs, int w, int h)
+{
+    std::vector<MarchCta> v;
+    for (int k = 0; k < count; ++k)
+        for (int y0 = 0; y0 < probs[k].ny; y0 += h)
+            for (int x0 = 0; x0 < probs[k].nx; x0 += w) v.push_back(MarchCta{k, x0, y0, std::min(h, probs[k].ny - y0)});
+    return v;
+}
+
+// One step of a group by tiles.
+template <typename T, int N>
+cudaError_t tiles_launch(const BatchGroup<T>* g, int parity, cudaStream_t st)
+{
+    if constexpr (std::is_same<T, float>::value && N <= ROWS_NMAX) {
+        kb_rows<N><<<g->ntiles, 32 * ROWS_WPC * N, 0, st>>>(g->mitems, g->tiles, parity);
+        return cudaGetLastError();
+    }
+    if constexpr (std::is_same<T, double>::value) {
+        const int threads = N * (g->ty << g->lx);
+        kb_tile_rho<N><<<g->ntiles, threads, 0, st>>>(g->mitems, g->tiles, parity, g->lx, g->ty);
+        kb_tile<N><<<g->ntiles, threads, sizeof(double) * tile_smem_values(N, 1 << g->lx, g->ty, false), st>>>(
+            g->mitems, g->tiles, parity, g->lx, g->ty);
+        return cudaGetLastError();
+    }
+    return cudaErrorInvalidValue;
 }
 
 // Kernel attributes of one geometry's batched march; *per_sm receives its resident CTAs.
@@ -244,6 +357,7 @@ bool march_group_create(BatchGroup<T>* g, int count, const Problem* probs, const
         items[k].p = make_params<C>(probs[k], scs[k].status);
         items[k].f[0] = static_cast<T*>(fa[k]);
         items[k].f[1] = static_cast<T*>(fb[k]);
+        items[k].rs = static_cast<C*>(scs[k].rho_s);
         const long long lines = (long long)N * probs[k].ny * (Q + (Storage<T>::shifted ? 1 : 0));
         gstart[k + 1] = gstart[k] + lines * 2 * probs[k].hx;
         const long long nb = (gstart[k + 1] - gstart[k] + 255) / 256;
@@ -269,6 +383,27 @@ bool march_group_create(BatchGroup<T>* g, int count, const Problem* probs, const
         if (narrow && !march_add_candidates<T, N, MarchNarrow<T, N>>(g, 1, count, probs,
                                                                    per_sm2 * std::max(1, sm_count), st))
             return false;
+    std::vector<MarchCta> tiles;
+    if (batch_takes_tiles<T>(N, count, probs)) {
+        if (std::is_same<T, double>::value) {
+            long long sites = 0;
+            for (int k = 0; k < count; ++k) sites += probs[k].S;
+            const bool small = N >= 5 || sites < 12800;
+            g->lx = small ? 3 : 4;
+            g->ty = small ? 4 : 8;
+            tiles = tile_ctas(count, probs, 1 << g->lx, g->ty);
+        } else {
+            tiles = tile_ctas(count, probs, ROWS_X, BATCH_TILE_ROWS);
+        }
+        if (tiles.size() > (size_t)INT32_MAX ||
+            cudaMalloc(&g->tiles, sizeof(MarchCta) * tiles.size()) != cudaSuccess ||
+            cudaMemcpyAsync(g->tiles, tiles.data(), sizeof(MarchCta) * tiles.size(), cudaMemcpyHostToDevice, st) != cudaSuccess) {
+            cudaGetLastError();
+            return false;
+        }
+        g->ntiles = (int)tiles.size();
+        g->use_tiles = true;
+    }
     if (cudaStreamSynchronize(st) != cudaSuccess) {
         cudaGetLastError();
         return false;
@@ -393,6 +528,7 @@ template <typename T, int N>
 cudaError_t batch_group_step_n(const BatchGroup<T>* g, int parity, cudaStream_t st, int part)
 {
     if (g->march) {
+        if (g->use_tiles) return part == 0 ? tiles_launch<T, N>(g, parity, st) : cudaSuccess;
         if (part == 0) return march_launch<T, N>(g, g->pick, parity, st);
         kb_ghosts<T><<<g->gblocks, 256, 0, st>>>(g->mitems, g->gstart, g->gfirst, g->gblk2inst, parity, N);
         return cudaGetLastError();
@@ -425,7 +561,7 @@ template <typename T>
 cudaError_t batch_group_tune(void* group, int parity, cudaStream_t st)
 {
     auto* g = static_cast<BatchGroup<T>*>(group);
-    if (!g->march || g->tuned) return cudaSuccess;
+    if (!g->march || g->tuned || g->use_tiles) return cudaSuccess;
     switch (g->N) {
         case 1: return march_group_tune<T, 1>(g, parity, st);
         case 2: return march_group_tune<T, 2>(g, parity, st);
@@ -449,17 +585,19 @@ bool batch_group_force(void* group, int narrow, int waves)
         if (g->cand_geo[c] == (narrow ? 1 : 0) && g->cand_waves[c] == waves) {
             g->pick = (int)c;
             g->tuned = true;
+            g->use_tiles = false;
             return true;
         }
     return false;
 }
 
-// waves of the CTA table in use (0 for the staged schedule), plus 1000 when the narrow
-// strip geometry was picked
+// waves of the CTA table in use (0 for the staged schedule, 1 for the tiles), plus 1000 when the
+// narrow strip geometry was picked
 template <typename T>
 int batch_group_waves(const void* group)
 {
     const auto* g = static_cast<const BatchGroup<T>*>(group);
+    if (g->use_tiles) return 1;
     return g->march ? g->cand_waves[g->pick] + 1000 * g->cand_geo[g->pick] : 0;
 }
 
@@ -495,7 +633,9 @@ bool batch_narrow_boxes(int N, int* box_w, int* out_w)
 template <typename T>
 int batch_group_launches(const void* group)
 {
-    return static_cast<const BatchGroup<T>*>(group)->march ? 2 : 3;
+    const auto* g = static_cast<const BatchGroup<T>*>(group);
+    if (g->use_tiles) return std::is_same<T, double>::value ? 2 : 1;
+    return g->march ? 2 : 3;
 }
 
 template <typename T>
@@ -507,6 +647,7 @@ void batch_group_destroy(void* group)
     if (g->blk2inst) cudaFree(g->blk2inst);
     if (g->mitems) cudaFree(g->mitems);
     for (MarchCta* d : g->cand) cudaFree(d);
+    if (g->tiles) cudaFree(g->tiles);
     if (g->gstart) cudaFree(g->gstart);
     if (g->gfirst) cudaFree(g->gfirst);
     if (g->gblk2inst) cudaFree(g->gblk2inst);

@@ -27,6 +27,8 @@ constexpr int ROWS_EY = ROWS_Y + 4;
 constexpr int ROWS_NY = ROWS_Y + 2;
 constexpr int ROWS_MIN_NY = ROWS_EY;   // rows wrap at most once
 constexpr int ROWS_NMAX = 5;           // two CTAs of more warps do not fit an SM's registers
+// CTAs an SM is to hold: about 36 warps of 48 to 64 registers
+__host__ __device__ constexpr int rows_ctas(int n) { return n == 1 ? 8 : n == 2 ? 4 : n == 3 ? 3 : 2; }
 
 // rho^s, nu^s, j^s of N components and u, in floats
 __host__ __device__ constexpr int rows_smem_floats(int n)
@@ -78,10 +80,13 @@ __device__ __forceinline__ void collide_poly2(const StepParams<float>& p, const 
     put(6, pfma(om, mone, em));
 }
 
-// One timestep fin -> fout.  gridDim = (column tiles, row tiles), blockDim.x = 128 N.
+// One timestep fin -> fout of the tile at column x0, row y0; CTA of 128 N threads.  p may live in
+// parameter or shared memory.  Ends with threads past the collision at different points:
+// another tile may follow at once (its first barrier is behind every read of this one's arrays
+// that it overwrites).
 template <int N, bool WALLS>
-__global__ void __launch_bounds__(32 * ROWS_WPC * N, N == 5 ? 2 : 1)
-k_rows(const float* __restrict__ fin, float* __restrict__ fout, const __grid_constant__ StepParams<float> p)
+__device__ __forceinline__ void rows_tile(const float* __restrict__ fin, float* __restrict__ fout,
+                                          const StepParams<float>& p, const int x0, const int y0)
 {
     __shared__ float R[N][ROWS_EY][32];
     __shared__ float NU[N][ROWS_NY][32];
@@ -90,7 +95,6 @@ k_rows(const float* __restrict__ fin, float* __restrict__ fout, const __grid_con
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int s = warp / ROWS_WPC, w = warp % ROWS_WPC;
-    const int x0 = blockIdx.x * ROWS_X, y0 = blockIdx.y * ROWS_Y;
     const int x = x0 - 2 + lane;
     const int ya = y0 + 2 * w;
     const unsigned pb = (unsigned)p.pitch * 4u, rb = Q * pb;   // bytes of a line and of a row
@@ -222,6 +226,14 @@ k_rows(const float* __restrict__ fin, float* __restrict__ fout, const __grid_con
             if (two) store_row(line_at(ob, pb, (unsigned)i) - (p.hx + x), x, p.nx, p.hx, out[i].y);
         }
     }
+}
+
+// gridDim = (column tiles, row tiles), blockDim.x = 128 N
+template <int N, bool WALLS>
+__global__ void __launch_bounds__(32 * ROWS_WPC * N, rows_ctas(N))
+k_rows(const float* __restrict__ fin, float* __restrict__ fout, const __grid_constant__ StepParams<float> p)
+{
+    rows_tile<N, WALLS>(fin, fout, p, blockIdx.x * ROWS_X, blockIdx.y * ROWS_Y);
 }
 
 }  // namespace mclb

@@ -385,8 +385,10 @@ struct TileLaunch {
         if constexpr (std::is_same<T, float>::value) {
             if (pl.lx == 0)
                 MCLB_DISPATCH_N(P.N, {
-                    return launch_dependent(P.walls ? k_rows<NN, true> : k_rows<NN, false>,
-                                            dim3(pl.gx, pl.gy), pl.threads, 0, st, (const T*)fin, (T*)fout, p);
+                    if constexpr (NN <= ROWS_NMAX)
+                        return launch_dependent(P.walls ? k_rows<NN, true> : k_rows<NN, false>,
+                                                dim3(pl.gx, pl.gy), pl.threads, 0, st, (const T*)fin, (T*)fout, p);
+                    return cudaErrorInvalidValue;
                 });
         }
         MCLB_DISPATCH_N(P.N, {

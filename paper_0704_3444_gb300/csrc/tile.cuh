@@ -193,15 +193,16 @@ k_tile_rho(const T* __restrict__ f, typename Storage<T>::C* __restrict__ rs,
     grid_dependents_launch();
 }
 
-// One timestep fin -> fout on the tiles blockIdx: columns [TX bx, ...), rows [y0, y0 + TY) with
-// y0 = TY by, TX = 1 << lx.  blockDim.x = N TX TY, or more: threads beyond those pull around the
-// tile while the others pull the tile, and parts > 1 spreads a site's potentials over as many
-// threads -- for tiles of so few warps that SM quarters would idle.  rs: the rho^s field of
-// fin, read around the tile instead of pulling there, or null.
+// One timestep fin -> fout on the tile at column x0, row y0: TX = 1 << lx columns, ty rows.
+// blockDim.x = N TX TY, or in FP64 more: threads beyond those pull around the tile while the
+// others pull the tile, and parts > 1 spreads a site's potentials over as many threads -- for
+// tiles of so few warps that SM quarters would idle.  rs: the rho^s field of fin, read around
+// the tile instead of pulling there, or null.  p may live in parameter or shared memory.
 template <typename T, int N>
-__global__ void __launch_bounds__(tile_max_threads<T>()) __maxnreg__(tile_max_regs<T>(N))
-k_tile(const T* __restrict__ fin, T* __restrict__ fout, const typename Storage<T>::C* __restrict__ rs,
-       const __grid_constant__ StepParams<typename Storage<T>::C> p, int lx, int ty, int parts64)
+__device__ __forceinline__ void tile_step(const T* __restrict__ fin, T* __restrict__ fout,
+                                          const typename Storage<T>::C* __restrict__ rs,
+                                          const StepParams<typename Storage<T>::C>& p, const int x0,
+                                          const int y0, int lx, int ty, int parts64)
 {
     using C = typename Storage<T>::C;
     constexpr bool F64 = sizeof(C) == 8;
@@ -222,7 +223,6 @@ k_tile(const T* __restrict__ fin, T* __restrict__ fout, const typename Storage<T
     const int s = tid / SITES, site = tid - s * SITES;
     const bool mine = !F64 || s < N;   // (else a thread beyond the tile's)
     const int tx = site & (TX - 1), tyy = site >> lx;
-    const int x0 = blockIdx.x << lx, y0 = blockIdx.y * ty;
     const int x = x0 + tx, y = y0 + tyy;
     const bool own = x < p.nx && y < p.ny;
     // (lanes beyond the lattice compute some site's values and store nothing)
@@ -395,6 +395,14 @@ k_tile(const T* __restrict__ fin, T* __restrict__ fout, const typename Storage<T
 #pragma unroll
         for (int i = 0; i < Q; ++i) put(row + i * (unsigned)p.pitch, out[i]);
     }
+}
+
+template <typename T, int N>
+__global__ void __launch_bounds__(tile_max_threads<T>()) __maxnreg__(tile_max_regs<T>(N))
+k_tile(const T* __restrict__ fin, T* __restrict__ fout, const typename Storage<T>::C* __restrict__ rs,
+       const __grid_constant__ StepParams<typename Storage<T>::C> p, int lx, int ty, int parts)
+{
+    tile_step<T, N>(fin, fout, rs, p, blockIdx.x << lx, blockIdx.y * ty, lx, ty, parts);
 }
 
 }  // namespace mclb

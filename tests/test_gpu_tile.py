@@ -125,3 +125,37 @@ def test_resume_and_non_finite(precision, shape):
     sim.step_nocheck(1)
     assert sim.status() == -4
     sim.close()
+
+
+def test_fp32_batch_by_row_tiles():
+    """FP32 batches large enough for the row tiles: instances narrower than a tile, at exact
+    multiples and with remainders, two groups side by side, an odd and an even number of
+    steps; densities and U within the FP32 tolerance of the oracle (1e-5) after 41 steps,
+    and the march takes over the same state from the tiles' ghost columns."""
+    probs = []
+    for k, (nx, ny, n) in enumerate([(700, 500, 2), (28, 12, 2), (421, 403, 2), (650, 433, 3), (57, 16, 3), (280, 240, 3)]):
+        rho, u = inputs.random_state(n, nx, ny, seed=640 + k, amp=0.1, umax=0.03)
+        p = inputs.Problem(name=f"r{k}", ncomp=n, nx=nx, ny=ny, tau=0.7 + 0.1 * k, chi=inputs.uniform_chi(n, 1.7),
+                           m=np.ones(n), theta=1 / 3, kappa=0.01, force=(1e-5, 0.0), rho=rho, u=u)
+        p.forcing_velocity = k % 2
+        probs.append(p)
+    b = mclb.Batch(probs, precision="fp32")
+    b.init_all()
+    b.step(1)
+    assert [w for _, w in b.tuning()] == [1, 1] and b.launches_per_step == 2
+    b.step(40)
+    assert b.status()[0] == 0
+    oracles = []
+    for k, p in enumerate(probs):
+        orc = Oracle.from_problem(p)
+        orc.run(41)
+        oracles.append(orc)
+        got, want = b.moments(k), orc.moments()
+        for f in ("rho", "U"):
+            assert np.max(np.abs(got[f] - want[f])) < 1e-5, (k, f)
+    assert b.test_force_partition(False, 4) == 2
+    b.step(3)
+    for k in (1, 4, 5):
+        oracles[k].run(3)
+        assert np.max(np.abs(b.moments(k)["rho"] - oracles[k].moments()["rho"])) < 1e-5, k
+    b.close()
