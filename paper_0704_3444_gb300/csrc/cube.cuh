@@ -148,13 +148,15 @@ __device__ __forceinline__ typename Storage<T>::C pull19(const T* __restrict__ f
     return Storage<T>::load(f + (long long)s * Q19 * p.S + at19(p, i, n.row, n.x));
 }
 
-// rho^s and, when js is given, the momenta j^s = sum_i f^s_i v_i ([s][d][site]) that the
+// rho^s and, when `total` is given, the total momentum ([d][site], for the output fields); when js
+// is given, the momenta j^s = sum_i f^s_i v_i ([s][d][site]) that the
 // collision would otherwise pull the populations a second time to form.
 template <typename T, int N>
 __global__ void __launch_bounds__(SITE_THREADS)
 k19_density(const T* __restrict__ f, typename Storage<T>::C* __restrict__ rs,
             typename Storage<T>::C* __restrict__ js,
-            const __grid_constant__ StepParams<typename Storage<T>::C> p)
+            const __grid_constant__ StepParams<typename Storage<T>::C> p,
+            double* __restrict__ total = nullptr)
 {
     using C = typename Storage<T>::C;
     const long long site = (long long)blockIdx.x * blockDim.x + threadIdx.x;
@@ -183,6 +185,14 @@ k19_density(const T* __restrict__ f, typename Storage<T>::C* __restrict__ rs,
         for (int s = 0; s < N; ++s)
 #pragma unroll
             for (int d = 0; d < 3; ++d) js[(s * 3 + d) * p.S + site] = j[s][d];
+    if (total)
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            C t = C(0);
+#pragma unroll
+            for (int s = 0; s < N; ++s) t += j[s][d];
+            stash1(total + d * p.S + site, t);
+        }
 }
 
 // lap g = 6 sum_i w_i (g(r + v_i) - g(r)) of every component's density field (each
@@ -442,14 +452,12 @@ k19_set_state(const double* __restrict__ in, T* __restrict__ f,
 // Output fields (after k19_density and k19_potential of the same state): rho^s; U (3 * S)
 // = u + (sum_s rho^s a^s)/(2 rho) (Eq. scon); mu^s; P (6 * S: xx, xy, xz, yy, yz, zz) =
 // (sum_s rho^s mu^s - psi) I + kappa sum_s grad rho^s grad rho^s (Eq. ppp, diagnostic).
-template <typename T, int N>
+template <typename C, int N>
 __global__ void __launch_bounds__(SITE_THREADS)
-k19_moments(const T* __restrict__ f, const typename Storage<T>::C* __restrict__ rs,
-            const typename Storage<T>::C* __restrict__ nu, double* __restrict__ rho_out,
+k19_moments(const C* __restrict__ rs, const C* __restrict__ nu, double* __restrict__ rho_out,
             double* __restrict__ U, double* __restrict__ mu_out, double* __restrict__ P,
-            const __grid_constant__ StepParams<typename Storage<T>::C> p)
+            const __grid_constant__ StepParams<C> p)
 {
-    using C = typename Storage<T>::C;
     const long long site = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (site >= p.S) return;
     const Site3 c = site3(p, site);
@@ -462,24 +470,19 @@ k19_moments(const T* __restrict__ f, const typename Storage<T>::C* __restrict__ 
     }
     if (rho_out)
 #pragma unroll
-        for (int s = 0; s < N; ++s) rho_out[s * p.S + site] = (double)r[s];
+        for (int s = 0; s < N; ++s) rho_out[s * p.S + site] = widen(r[s]);
     if (U) {
-        C jt[3] = {C(0), C(0), C(0)}, ft[3] = {C(0), C(0), C(0)};
+        // U holds the total momentum (k19_density)
+        C ft[3] = {C(0), C(0), C(0)};
         C a[N][3];
         accel19<C, N>(rs, nu, p, c, r, rho, a);
 #pragma unroll
-        for (int s = 0; s < N; ++s) {
-#pragma unroll
-            for (int i = 0; i < Q19; ++i) {
-                const C v = pull19(f, p, s, i, c);
-#pragma unroll
-                for (int d = 0; d < 3; ++d) jt[d] += v * C(c19(i, d));
-            }
+        for (int s = 0; s < N; ++s)
 #pragma unroll
             for (int d = 0; d < 3; ++d) ft[d] += r[s] * a[s][d];
-        }
 #pragma unroll
-        for (int d = 0; d < 3; ++d) U[d * p.S + site] = (double)(jt[d] / rho + C(0.5) * ft[d] / rho);
+        for (int d = 0; d < 3; ++d)
+            U[d * p.S + site] = widen(fma(C(0.5), ft[d], unstash1<C>(U + d * p.S + site)) / rho);
     }
     if (mu_out || P) {
         C lap[N], mu[N];
@@ -487,7 +490,7 @@ k19_moments(const T* __restrict__ f, const typename Storage<T>::C* __restrict__ 
         site_mu<C, N>(p, r, lap, mu);
         if (mu_out)
 #pragma unroll
-            for (int s = 0; s < N; ++s) mu_out[s * p.S + site] = (double)mu[s];
+            for (int s = 0; s < N; ++s) mu_out[s * p.S + site] = widen(mu[s]);
         if (P) {
             const C psi = site_psi<C, N>(p, r);
             C rmu = C(0), gg = C(0), t[6] = {C(0), C(0), C(0), C(0), C(0), C(0)};
@@ -505,12 +508,12 @@ k19_moments(const T* __restrict__ f, const typename Storage<T>::C* __restrict__ 
                 t[5] += p.kappa * g[2] * g[2];
             }
             const C iso = rmu - (psi + gg);
-            P[site] = (double)(iso + t[0]);
-            P[p.S + site] = (double)t[1];
-            P[2 * p.S + site] = (double)t[2];
-            P[3 * p.S + site] = (double)(iso + t[3]);
-            P[4 * p.S + site] = (double)t[4];
-            P[5 * p.S + site] = (double)(iso + t[5]);
+            P[site] = widen(iso + t[0]);
+            P[p.S + site] = widen(t[1]);
+            P[2 * p.S + site] = widen(t[2]);
+            P[3 * p.S + site] = widen(iso + t[3]);
+            P[4 * p.S + site] = widen(t[4]);
+            P[5 * p.S + site] = widen(iso + t[5]);
         }
     }
 }

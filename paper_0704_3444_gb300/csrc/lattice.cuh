@@ -170,6 +170,61 @@ inline StepParams<C> make_params(const Problem& P, unsigned int* status)
     return p;
 }
 
+// The double of the same value.  The conversion instruction runs in the FP64 pipe, 64 cycles per
+// warp and SM quarter (measured); the output fields of an FP32 state are millions of them, so the
+// bits are moved instead: the exponent rebiased, the fraction shifted.
+__device__ __forceinline__ double widen(double v) { return v; }
+__device__ __forceinline__ double widen(float v)
+{
+    const unsigned b = __float_as_uint(v), a = b & 0x7fffffffu, sign = b & 0x80000000u;
+    unsigned hi = (a >> 3) + (896u << 20), lo = b << 29;
+    if (a - 0x00800000u >= 0x7f000000u) {   // zero, subnormal, infinite or NaN
+        if (a == 0) {
+            hi = 0;
+        } else if (a >= 0x7f800000u) {
+            hi = 0x7ff00000u | ((a & 0x007fffffu) >> 3);
+        } else {
+            const unsigned n = __float_as_uint(v * 0x1p24f) & 0x7fffffffu;   // normal, exact
+            hi = (n >> 3) + ((896u - 24u) << 20);
+            lo = n << 29;
+        }
+    }
+    return __hiloint2double((int)(hi | sign), (int)lo);
+}
+
+// Values of C kept in an output array until the pass that overwrites them: one in a double's
+// place; two in one double's place (FP32) or in q[0] and q[S] (FP64).
+template <typename C>
+__device__ __forceinline__ void stash1(double* q, C v) { *reinterpret_cast<C*>(q) = v; }
+template <typename C>
+__device__ __forceinline__ C unstash1(const double* q) { return *reinterpret_cast<const C*>(q); }
+__device__ __forceinline__ void stash2(double* q, long long, float a, float b)
+{
+    *reinterpret_cast<float2*>(q) = make_float2(a, b);
+}
+__device__ __forceinline__ void stash2(double* q, long long S, double a, double b)
+{
+    q[0] = a;
+    q[S] = b;
+}
+__device__ __forceinline__ void unstash2(const double* q, long long, float& a, float& b)
+{
+    const float2 v = *reinterpret_cast<const float2*>(q);
+    a = v.x;
+    b = v.y;
+}
+__device__ __forceinline__ void unstash2(const double* q, long long S, double& a, double& b)
+{
+    a = q[0];
+    b = q[S];
+}
+
+// Programmatic dependent launch: wait until the kernels this one depends on are complete and
+// their writes visible; let the next kernel of the stream be scheduled (its own wait still
+// covers this one's end).
+__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_dependents_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // a + d mod n for |d| <= n
 __device__ __forceinline__ int wrap_add(int a, int d, int n)
 {

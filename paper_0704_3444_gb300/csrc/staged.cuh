@@ -84,29 +84,40 @@ __device__ __forceinline__ bool bounced(const StepParams<C>& p, int y, int i)
     return p.walls && (yy < 0 || yy >= p.ny);
 }
 
-// rho^s at one site (pull streaming + zeroth moment).
+// rho^s at one site (pull streaming + zeroth moment) and, when j (the output U) is given, the
+// total momentum sum_s j^s stashed at the site.
 template <typename T, int N, bool E = true>
 __device__ __forceinline__ void density_site(const T* __restrict__ f,
                                              typename Storage<T>::C* __restrict__ rs,
-                                             const StepParams<typename Storage<T>::C>& p, long long site)
+                                             const StepParams<typename Storage<T>::C>& p, long long site,
+                                             double* __restrict__ j = nullptr)
 {
     using C = typename Storage<T>::C;
     const int y = (int)(site / p.nx), x = (int)(site - (long long)y * p.nx);
+    C jx = C(0), jy = C(0);
 #pragma unroll
     for (int s = 0; s < N; ++s) {
         C r = C(0);
 #pragma unroll
-        for (int i = 0; i < Q; ++i) r += pull<E>(f, p, s, i, x, y);
+        for (int i = 0; i < Q; ++i) {
+            const C v = pull<E>(f, p, s, i, x, y);
+            r += v;
+            jx += v * C(vx(i));
+            jy += v * C(vy(i));
+        }
         rs[s * p.S + site] = r;
     }
+    if (j) stash2(j + site, p.S, jx, jy);
 }
 
 template <typename T, int N, bool BAND = false>
 __global__ void __launch_bounds__(SITE_THREADS)
 k_density(const T* __restrict__ f, typename Storage<T>::C* __restrict__ rs,
-          const __grid_constant__ StepParams<typename Storage<T>::C> p)
+          const __grid_constant__ StepParams<typename Storage<T>::C> p, double* __restrict__ j = nullptr)
 {
     long long site = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    grid_dependency_wait();
+    grid_dependents_launch();
     if constexpr (BAND) {
         site = site_of(p, site);
         if (site < 0) return;
@@ -114,9 +125,9 @@ k_density(const T* __restrict__ f, typename Storage<T>::C* __restrict__ rs,
         return;
     }
     if (wall_row(p, site))
-        density_site<T, N, true>(f, rs, p, site);
+        density_site<T, N, true>(f, rs, p, site, BAND ? nullptr : j);
     else
-        density_site<T, N, false>(f, rs, p, site);
+        density_site<T, N, false>(f, rs, p, site, BAND ? nullptr : j);
 }
 
 template <typename C, int N, bool E = true>
@@ -362,75 +373,6 @@ k_set_state(const double* __restrict__ in, T* __restrict__ f,
     }
 #pragma unroll
     for (int s = 0; s < N; ++s) store_site(f, p, s, y, x, v[s]);
-}
-
-// Output fields: rho^s, U = u + (sum_s rho^s a^s)/(2 rho), mu^s, P (needs k_density and
-// k_potential to have filled the scratch fields for the same state).
-template <typename T, int N>
-__global__ void __launch_bounds__(SITE_THREADS)
-k_moments(const T* __restrict__ f, const typename Storage<T>::C* __restrict__ rs,
-          const typename Storage<T>::C* __restrict__ nu, double* __restrict__ rho_out,
-          double* __restrict__ U, double* __restrict__ mu_out, double* __restrict__ P,
-          const __grid_constant__ StepParams<typename Storage<T>::C> p)
-{
-    using C = typename Storage<T>::C;
-    const long long site = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    if (site >= p.S) return;
-    const int y = (int)(site / p.nx), x = (int)(site - (long long)y * p.nx);
-    C r[N];
-    C rho = C(0);
-#pragma unroll
-    for (int s = 0; s < N; ++s) {
-        r[s] = rs[s * p.S + site];
-        rho += r[s];
-    }
-    if (rho_out)
-#pragma unroll
-        for (int s = 0; s < N; ++s) rho_out[s * p.S + site] = (double)r[s];
-    if (U) {
-        C jxt = C(0), jyt = C(0), fx = C(0), fy = C(0);
-        C ax[N], ay[N];
-        site_accel<C, N>(rs, nu, p, x, y, r, rho, ax, ay);
-#pragma unroll
-        for (int s = 0; s < N; ++s) {
-#pragma unroll
-            for (int i = 0; i < Q; ++i) {
-                const C v = pull(f, p, s, i, x, y);
-                jxt += v * C(vx(i));
-                jyt += v * C(vy(i));
-            }
-            fx += r[s] * ax[s];
-            fy += r[s] * ay[s];
-        }
-        U[site] = (double)(jxt / rho + C(0.5) * fx / rho);
-        U[p.S + site] = (double)(jyt / rho + C(0.5) * fy / rho);
-    }
-    if (mu_out || P) {
-        C lap[N], mu[N];
-        neighbour_laplacians<C, N>(rs, p, x, y, r, lap);
-        site_mu<C, N>(p, r, lap, mu);
-        if (mu_out)
-#pragma unroll
-            for (int s = 0; s < N; ++s) mu_out[s * p.S + site] = (double)mu[s];
-        if (P) {
-            const C psi = site_psi<C, N>(p, r);
-            C rmu = C(0), gg = C(0), pxx = C(0), pxy = C(0), pyy = C(0);
-#pragma unroll
-            for (int s = 0; s < N; ++s) {
-                C gx, gy;
-                field_grad(rs + s * p.S, p, x, y, gx, gy);
-                rmu += r[s] * mu[s];
-                gg += C(0.5) * p.kappa * (gx * gx + gy * gy);
-                pxx += p.kappa * gx * gx;
-                pxy += p.kappa * gx * gy;
-                pyy += p.kappa * gy * gy;
-            }
-            const C iso = rmu - (psi + gg);
-            P[site] = (double)(iso + pxx);
-            P[p.S + site] = (double)pxy;
-            P[2 * p.S + site] = (double)(iso + pyy);
-        }
-    }
 }
 
 // Deterministic FP64 block reduction of K values per thread into partial[block * K + k].

@@ -6,6 +6,7 @@
 #include "batch.cuh"
 #include "cube.cuh"
 #include "cube_march.cuh"
+#include "fields.cuh"
 #include "ghosts.cuh"
 #include "line3.cuh"
 #include "march.cuh"
@@ -30,6 +31,25 @@ namespace mclb {
     }
 
 inline unsigned site_blocks(long long S) { return (unsigned)((S + SITE_THREADS - 1) / SITE_THREADS); }
+
+// Launch with programmatic stream serialisation: the kernel may be scheduled while the one
+// before it drains (it waits for that one's end itself).
+template <typename... P, typename... A>
+cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st,
+                             A... args)
+{
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
+}
 
 template <typename T>
 struct Launch {
@@ -195,12 +215,26 @@ struct Launch {
                                double* U, double* mu, double* Pt, cudaStream_t st)
     {
         const auto p = make_params<C>(P, sc.status);
+        // Tiles of 14 rows by eight warps: potentials on 16 rows, two a warp.  Six where their
+        // shared memory does not fit; two by four warps where the larger ones would leave SMs
+        // without one (and FP64 its pipe on those).
+        int rows = 14, warps = FIELDS_MAX_WARPS;
+        const auto smem = [&](int r) { return sizeof(C) * fields_smem_values(P.N, r); };
+        if (smem(rows) > 44 * 1024) rows = 6;
+        if (P.S < 152LL * FIELDS_X * rows) {
+            rows = 2;
+            warps = 4;
+        }
+        const long long tiles = (long long)((P.nx + FIELDS_X - 1) / FIELDS_X) * ((P.ny + rows - 1) / rows);
+        const dim3 grid((unsigned)tiles);   // (at most the 2^31 sites' number)
         MCLB_DISPATCH_N(P.N, {
-            cudaError_t e = fields_n<NN>(p, sc, (const T*)f, st);
+            // (few sites: smaller blocks, so that every SM has one)
+            const int dt = P.S < 152LL * SITE_THREADS ? 64 : SITE_THREADS;
+            cudaError_t e = launch_dependent(k_density<T, NN, false>, dim3((unsigned)((P.S + dt - 1) / dt)), dt,
+                                             0, st, (const T*)f, (C*)sc.rho_s, p, U);
             if (e != cudaSuccess) return e;
-            k_moments<T, NN><<<site_blocks(P.S), SITE_THREADS, 0, st>>>(
-                (const T*)f, (const C*)sc.rho_s, (const C*)sc.nu, rho, U, mu, Pt, p);
-            return cudaGetLastError();
+            return launch_dependent(k_fields<C, NN>, grid, 32 * warps, smem(rows), st, (const C*)sc.rho_s, rho,
+                                    U, mu, Pt, p, rows);
         });
     }
 
@@ -284,25 +318,6 @@ struct Launch {
         return cudaGetLastError();
     }
 };
-
-// Launch with programmatic stream serialisation: the kernel may be scheduled while the one
-// before it drains (it waits for that one's end itself).
-template <typename... P, typename... A>
-cudaError_t launch_dependent(void (*kern)(P...), dim3 grid, int threads, size_t smem, cudaStream_t st,
-                             A... args)
-{
-    cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3((unsigned)threads);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kern, static_cast<P>(args)...);
-}
 
 // The tile schedule (tile.cuh) for one storage type.
 template <typename T>
@@ -821,10 +836,13 @@ struct Launch19 {
     {
         const auto p = make_params<C>(P, sc.status);
         MCLB_DISPATCH_N(P.N, {
-            cudaError_t e = fields_n<NN>(p, sc, (const T*)f, st);
-            if (e != cudaSuccess) return e;
-            k19_moments<T, NN><<<site_blocks(P.S), SITE_THREADS, 0, st>>>(
-                (const T*)f, (const C*)sc.rho_s, (const C*)sc.nu, rho, U, mu, Pt, p);
+            k19_density<T, NN><<<site_blocks(P.S), SITE_THREADS, 0, st>>>((const T*)f, (C*)sc.rho_s,
+                                                                          nullptr, p, U);
+            if (U)
+                k19_potential<C, NN><<<site_blocks(P.S), SITE_THREADS, 0, st>>>((const C*)sc.rho_s,
+                                                                                (C*)sc.nu, p);
+            k19_moments<C, NN><<<site_blocks(P.S), SITE_THREADS, 0, st>>>(
+                (const C*)sc.rho_s, (const C*)sc.nu, rho, U, mu, Pt, p);
             return cudaGetLastError();
         });
     }

@@ -32,12 +32,6 @@ constexpr int tile_max_threads() { return sizeof(typename Storage<T>::C) == 8 ? 
 template <typename T>
 constexpr int tile_max_regs(int n) { return sizeof(typename Storage<T>::C) == 8 ? (n <= 4 ? 80 : 128) : 56; }
 
-// Programmatic dependent launch: wait until the kernels this one depends on are complete and
-// their writes visible; let the next kernel of the stream be scheduled (its own wait still
-// covers this one's end).
-__device__ __forceinline__ void grid_dependency_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_dependents_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // Shared memory of one CTA in values of C: rho^s, nu^s, j^s, u and (Gibbs-Duhem) rho, 1/rho, a^s.
 __host__ __device__ constexpr int tile_smem_values(int n, int tx, int ty, bool gd)
 {
