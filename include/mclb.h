@@ -155,8 +155,8 @@ typedef enum {
  *              images of the rows next to it (zero normal gradient: neutral wetting).
  *              x stays periodic.  D2Q9 only; both schedules: the single pass computes
  *              every row at least three rows from a wall (their update reaches no row
- *              beyond one) and three staged launches then redo the rows next to the
- *              walls.  Single handles only (batches and mclb_step_noalloc reject it)
+ *              beyond one) and three staged launches, or with kernel AUTO one launch
+ *              of small tiles, then redo the rows next to the walls.  Single handles only (batches and mclb_step_noalloc reject it)
  *   mass_every 0 (off, the default) or the period, in timesteps, of the per-component
  *              mass compensation.  Eq. ff1 and the collision keep every component's total
  *              mass exactly; stored in FP32 or 16 bits, the rounding of each site's
@@ -327,8 +327,9 @@ int mclb_test_withhold_copies(mclb_handle h, int on);
 double mclb_bytes_per_step(mclb_handle h);
 
 /* Kernel launches one timestep issues (2 for the fused schedule: the single pass and
- * the refresh of the periodic ghost columns; 3 for the staged; 1 for the small tiles AUTO
- * may pick, 2 with the Gibbs-Duhem form; 1 on D1Q3, where one launch advances a resident
+ * the refresh of the periodic ghost columns, between walls 3 more, or with AUTO 1 more, for the
+ * rows next to them; 3 for the staged; 1 for the small tiles AUTO may pick, 2 with the
+ * Gibbs-Duhem form; 1 on D1Q3, where one launch advances a resident
  * line by up to 4096 timesteps). */
 int mclb_launches_per_step(mclb_handle h);
 

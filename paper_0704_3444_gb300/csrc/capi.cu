@@ -515,7 +515,10 @@ int mclb_create(const mclb_params* params, mclb_handle* out)
         if (h->plan.ok && make_tmap(h, 0) == MCLB_OK && make_tmap(h, 1) == MCLB_OK) h->fused = true;
         if (!h->fused && h->kernel == MCLB_KERNEL_FUSED)
             return bail(fail(MCLB_EINVAL, "fused kernel unavailable for this problem"));
-        if (h->kernel == MCLB_KERNEL_AUTO && h->fused) h->tile = h->tab->plan_tile(P, sms);
+        if (h->kernel == MCLB_KERNEL_AUTO && h->fused) {
+            h->tile = h->tab->plan_tile(P, sms);
+            h->plan.wall_tiles = h->tab->wall_tiles_fit(P);
+        }
     }
     cudaGetLastError();
     if (cudaStreamSynchronize(h->stream) != cudaSuccess)   // the zeroed buffers and status
@@ -678,6 +681,7 @@ int mclb_launches_per_step(mclb_handle h)
     if (h->P.lattice == MCLB_D1Q3) return 1;
     if (h->P.lattice == MCLB_D3Q19) return h->fused ? 2 : 3;   // density + march, or staged
     if (h->tile.ok) return h->P.force_form == FORCE_GIBBS_DUHEM ? 2 : 1;
+    if (h->fused && h->plan.wall_tiles) return 3;   // k_march, k_ghosts, the rows next to the walls
     if (h->fused) return h->P.walls ? 5 : 2;   // k_march, k_ghosts (+ three wall-row launches)
     return 3;
 }

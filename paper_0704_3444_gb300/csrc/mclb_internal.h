@@ -80,6 +80,7 @@ struct FusedPlan {
     int nstrips, nsegs;
     int threads;
     size_t smem;
+    bool wall_tiles;        // between walls: the rows next to them by one tile launch
     bool ok;
 };
 
@@ -139,6 +140,7 @@ struct KernelTable {
     CUtensorMapDataType tma_type;
     int hx;                 // ghost columns per side for this storage type
     FusedPlan (*plan_fused)(const Problem&, int sm_count);
+    bool (*wall_tiles_fit)(const Problem&);
     // f^s_i(r) = equilibrium of (rho, u) (device FP64 inputs; u may be null)
     cudaError_t (*init)(const Problem&, const Scratch&, const double* rho, const double* u,
                         void* f, cudaStream_t st);

@@ -115,6 +115,7 @@ struct Launch {
         pl.out_w = G::TMA_STORE ? MARCH_OUT : (G::CTA_STORE ? G::WOUT : 0);
         pl.NS = G::STAGES;
         pl.smem = G::SMEM;
+        pl.wall_tiles = false;
         pl.threads = G::THREADS;
         pl.nstrips = (P.nx + G::WOUT - 1) / G::WOUT;
         const int slots = ctas * std::max(1, sm_count);
@@ -183,6 +184,23 @@ struct Launch {
         return cudaGetLastError();
     }
 
+    // The same rows by one launch of tiles: us a step against the three band launches: 1500 x 1200 x 3
+    // FP32 80 / 95, 1024 x 2048 x 5 148 / 179, 1000 x 700 x 3 BF16 45.5 / 67.8.
+    static bool wall_tiles_fit(const Problem& P)
+    {
+        return P.walls && P.force_form == 0 && P.ny >= 2 * TILE_WALL_ROWS &&
+               P.N * 32 * TILE_WALL_ROWS <= tile_max_threads<T>() && (long long)P.plane * P.N < (1LL << 31);
+    }
+    template <int N>
+    static cudaError_t wall_tiles(const StepParams<C>& p, const T* fin, T* fout, cudaStream_t st)
+    {
+        if constexpr (N * 32 * TILE_WALL_ROWS <= tile_max_threads<T>()) {
+            return launch_dependent(k_tile_walls<T, N>, dim3((p.nx + 31) / 32, 2), N * 32 * TILE_WALL_ROWS,
+                                    sizeof(C) * tile_smem_values(N, 32, TILE_WALL_ROWS, false), st, fin, fout, p);
+        }
+        return cudaErrorInvalidValue;
+    }
+
     static cudaError_t step_fused(const Problem& P, const Scratch& sc, const FusedPlan& pl,
                                   const CUtensorMap* tmap_in, const CUtensorMap* tmapr_in,
                                   const CUtensorMap* tmapw_out, const CUtensorMap* tmapwr_out,
@@ -206,8 +224,9 @@ struct Launch {
                 k_march<T, NN><<<grid, pl.threads, pl.smem, st>>>(*tmap_in, tr, tw, twr, (T*)fout, p, pl.H);
             const long long ghosts = (long long)NN * P.ny * (Q + (Storage<T>::shifted ? 1 : 0)) * 2 * P.hx;
             k_ghosts<T><<<(unsigned)((ghosts + 255) / 256), 256, 0, st>>>((T*)fout, p, NN);
-            if (P.walls) return wall_rows<NN>(p, sc, (const T*)fin, (T*)fout, st);
-            return cudaGetLastError();
+            if (!P.walls) return cudaGetLastError();
+            if (pl.wall_tiles) return wall_tiles<NN>(p, (const T*)fin, (T*)fout, st);
+            return wall_rows<NN>(p, sc, (const T*)fin, (T*)fout, st);
         });
     }
 
@@ -325,25 +344,24 @@ struct TileLaunch {
     using C = typename Storage<T>::C;
 
     // Most sites x components for which a tile kernel beats the march (measured on both sides of
-    // each line, us per step, tile / march; between walls the march also pays three band
-    // launches, about 20 us):
+    // each line, us per step, tile / march; between walls the march has one launch more):
     //   FP64: it runs at the FP64 pipe's rate on every SM with fewer FP64 instructions a site:
     //     64 x 64 x 2 9.73 / 107, 2048^2 x 2 2323 / 2613, 2048^2 x 3 3474 / 3802, 600^2 x 6 758 /
     //     1233, 500^2 x 8 714 / 1130, Gibbs-Duhem 1024^2 x 3 967 / 1132: every size, but
     //     1024^2 x 4 1270 / 1230, 1024^2 x 5 1640 / 1494
     //   FP32 (k_rows): 1000^2 x 1 18.1 / 26.3; 700^2 x 2 20.5 / 22.3, 1024^2 x 2 38 / 37;
     //     512 x 384 x 3 14.7 / 18.5, 700 x 600 x 3 29.8 / 25.7; 400^2 x 4 21.7 / 20.1;
-    //     300^2 x 5 13.5 / 19.4, 500 x 450 x 5 24.9 / 23.6; walls 1000 x 333 x 3 21 / 39,
-    //     1500 x 1200 x 3 107 / 95.  k_tile, six and more: 300^2 x 6 20.0 / 23.1
-    //   16-bit: 400 x 300 x 4 19.7 / 22.8, 400^2 x 5 33 / 30; walls 1000 x 700 x 3 65.5 / 66.6
+    //     300^2 x 5 13.5 / 19.4, 500 x 450 x 5 24.9 / 23.6; walls 1000 x 333 x 3 21 / 31,
+    //     1500 x 1200 x 3 107 / 80.  k_tile, six and more: 300^2 x 6 20.0 / 23.1
+    //   16-bit: 400 x 300 x 4 19.7 / 22.8, 400^2 x 5 33 / 30; walls 1000 x 700 x 3 65.5 / 45.5
     //   FP32 Gibbs-Duhem: 300^2 x 2 10.3 / 15.8, 512 x 384 x 3 22.8 / 18.5
     static long long most(const Problem& P)
     {
         const int N = P.N;
         if (sizeof(C) == 8) return N == 4 || N == 5 ? 3000000 : 1LL << 40;
         if (P.force_form == FORCE_GIBBS_DUHEM) return 350000;
-        if (Storage<T>::shifted) return P.walls ? 2000000 : 600000;
-        if (P.walls) return 4000000;
+        if (Storage<T>::shifted) return P.walls ? 800000 : 600000;
+        if (P.walls) return 2500000;
         return N == 1 ? 2000000 : N == 2 ? 1200000 : N == 4 || N >= 6 ? 550000 : 900000;
     }
 
@@ -935,6 +953,7 @@ template <typename T>
 inline void fill_march(KernelTable& t)
 {
     t.plan_fused = &Launch<T>::plan_fused;
+    t.wall_tiles_fit = &Launch<T>::wall_tiles_fit;
     t.step_fused = &Launch<T>::step_fused;
 }
 

@@ -391,6 +391,18 @@ __device__ __forceinline__ void tile_step(const T* __restrict__ fin, T* __restri
     }
 }
 
+// The three rows next to each wall (blockIdx.y: the lower, the upper one), for a lattice whose
+// other rows the march steps: tiles of 32 x 3 sites.
+constexpr int TILE_WALL_ROWS = 3;
+template <typename T, int N>
+__global__ void __launch_bounds__(tile_max_threads<T>()) __maxnreg__(tile_max_regs<T>(N))
+k_tile_walls(const T* __restrict__ fin, T* __restrict__ fout,
+             const __grid_constant__ StepParams<typename Storage<T>::C> p)
+{
+    tile_step<T, N>(fin, fout, nullptr, p, blockIdx.x * 32, blockIdx.y ? p.ny - TILE_WALL_ROWS : 0, 5,
+                    TILE_WALL_ROWS, 1);
+}
+
 template <typename T, int N>
 __global__ void __launch_bounds__(tile_max_threads<T>()) __maxnreg__(tile_max_regs<T>(N))
 k_tile(const T* __restrict__ fin, T* __restrict__ fout, const typename Storage<T>::C* __restrict__ rs,

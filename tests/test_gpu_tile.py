@@ -159,3 +159,22 @@ def test_fp32_batch_by_row_tiles():
         oracles[k].run(3)
         assert np.max(np.abs(b.moments(k)["rho"] - oracles[k].moments()["rho"])) < 1e-5, k
     b.close()
+
+
+@pytest.mark.parametrize("precision,shape,steps", [("fp32", (1500, 601, 3), 10), ("bf16", (701, 420, 3), 10),
+                                                   ("fp64", (1003, 760, 4), 5), ("fp32", (420000, 6, 1), 6)],
+                         ids=lambda v: str(v))
+def test_march_between_walls_with_wall_tiles(precision, shape, steps):
+    """Lattices between walls that the march steps under AUTO: the rows next to the walls by one
+    tile launch; densities, U (and the FP64 state) to the formats' parity with the oracle."""
+    sim, orc = _pair(shape, precision, fv=1, walls=1, amp=0.1)
+    assert sim.launches_per_step == 3
+    sim.step(steps)
+    assert orc.run(steps) == 0
+    assert sim.status() == 0
+    got, want = sim.moments(mu=False, P=False), orc.moments()
+    tol = {"fp64": 1e-12, "fp32": 1e-5, "bf16": 2e-3}[precision]
+    assert np.max(np.abs(got["rho"] - want["rho"])) < tol and np.max(np.abs(got["U"] - want["U"])) < tol
+    if precision == "fp64":
+        assert _rel(sim.get_state(), orc.f) < 1e-12
+    sim.close()
