@@ -121,8 +121,9 @@ typedef enum {
                         handles only.  Kernel AUTO or FUSED: a density pass and a march
                         over z planes that forms the potentials on chip and collides (two
                         launches per step; N <= 4, Eq. definef as printed; FUSED fails
-                        with MCLB_EINVAL otherwise, AUTO falls back); STAGED: three
-                        launches.  The two schedules give the same values bit for bit.
+                        with MCLB_EINVAL otherwise, AUTO falls back, and takes it only
+                        where it is the faster one: FP32, N <= 3, from about 1e6
+                        site-components on); STAGED: three launches.  The two schedules give the same values bit for bit.
                         Fields are [.][z][y][x]; U has 3 components, P 6 (xx, xy, xz, yy,
                         yz, zz), the momentum and force sums 3                             */
 } mclb_lattice;

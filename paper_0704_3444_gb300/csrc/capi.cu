@@ -503,7 +503,8 @@ int mclb_create(const mclb_params* params, mclb_handle* out)
         if (h->alt->prepare(P, h->sc, h->f) != cudaSuccess ||
             cudaStreamSynchronize(cudaStreamLegacy) != cudaSuccess)
             return bail(fail(MCLB_ECUDA, "D1Q3 line description upload failed"));
-        if (h->alt->plan && h->kernel != MCLB_KERNEL_STAGED) {
+        const bool pays = h->kernel == MCLB_KERNEL_FUSED || !h->alt->pays || h->alt->pays(P);
+        if (h->alt->plan && h->kernel != MCLB_KERNEL_STAGED && pays) {
             const int r = h->alt->plan(h->P, sms);
             if (r < 0) return bail(fail(MCLB_ECUDA, "single-pass kernel set-up failed"));
             h->fused = r == 1;

@@ -148,9 +148,122 @@ __device__ __forceinline__ typename Storage<T>::C pull19(const T* __restrict__ f
     return Storage<T>::load(f + (long long)s * Q19 * p.S + at19(p, i, n.row, n.x));
 }
 
-// rho^s and, when `total` is given, the total momentum ([d][site], for the output fields); when js
-// is given, the momenta j^s = sum_i f^s_i v_i ([s][d][site]) that the
-// collision would otherwise pull the populations a second time to form.
+// The discrete operators over the eighteen neighbours and the collision, written once for the
+// staged kernels and the march (cube_march.cuh), whose states are equal bit for bit: sums of
+// sums and explicit fused multiply-adds, which leave the compiler no choice of contraction.
+
+// lap g = 6 sum_i w_i (g(r + v_i) - g(r)) = 1/3 (axis sum) + 1/6 (diagonal sum) - 4 g(r), from g(i) =
+// the neighbour's value (19 operations; difference by difference it takes 36)
+template <typename C, typename G>
+__device__ __forceinline__ C lap19(C g0, const G& g)
+{
+    const C ax = ((g(1) + g(2)) + (g(3) + g(4))) + (g(5) + g(6));
+    const C d1 = (g(7) + g(8)) + (g(9) + g(10)), d2 = (g(11) + g(12)) + (g(13) + g(14));
+    const C d3 = (g(15) + g(16)) + (g(17) + g(18));
+    return fma(C(1.0 / 3.0), ax, fma(C(1.0 / 6.0), (d1 + d2) + d3, C(-4) * g0));
+}
+
+// grad g = 3 sum_i w_i v_i g(r + v_i), from the nine differences of opposite neighbours
+template <typename C, typename G>
+__device__ __forceinline__ void gradient19(const G& g, C (&gr)[3])
+{
+    const C a = g(7) - g(8), b = g(9) - g(10), c = g(11) - g(12), d = g(13) - g(14);
+    const C e = g(15) - g(16), f = g(17) - g(18);
+    const C k1 = C(1.0 / 6.0), k2 = C(1.0 / 12.0);
+    gr[0] = fma(k1, g(1) - g(2), k2 * ((a + b) + (c + d)));
+    gr[1] = fma(k1, g(3) - g(4), k2 * ((a - b) + (e + f)));
+    gr[2] = fma(k1, g(5) - g(6), k2 * ((c - d) + (e - f)));
+}
+
+// j += the momentum of the opposite velocities 2k - 1 and 2k, whose populations differ by d (21
+// additions for the nine pairs, 30 velocity by velocity)
+template <typename C>
+__device__ __forceinline__ void add_momentum19(int k, C d, C (&j)[3])
+{
+    if (k <= 3)
+        j[k - 1] = d;
+    else if (k == 4 || k == 5) {
+        j[0] += d;
+        j[1] = k == 4 ? j[1] + d : j[1] - d;
+    } else if (k == 6 || k == 7) {
+        j[0] += d;
+        j[2] = k == 6 ? j[2] + d : j[2] - d;
+    } else {
+        j[1] += d;
+        j[2] = k == 8 ? j[2] + d : j[2] - d;
+    }
+}
+
+// The same as the velocities come one by one (held: f of the pair's first).  j starts at zero.
+template <typename C>
+__device__ __forceinline__ void momentum19(int i, C v, C& held, C (&j)[3])
+{
+    if (i & 1)
+        held = v;
+    else if (i > 0)
+        add_momentum19(i / 2, held - v, j);
+}
+
+// Post-collision values of one component (Eq. ssLB with the forcing of Eqs. ff1-ff3), two
+// opposite velocities at a time: with l = rho^s/tau u + rho^s a and, times 9,
+//   B_dd = rho^s/tau u_d^2/2 + a_d J_d,  B_de = rho^s/tau u_d u_e + a_d J_e + a_e J_d,
+//   f*_i = (1 - 1/tau) f_i + w_i [rho^s/tau + 9 (B:vv - tr B/3) + 3 l.v]
+// (the even part of a pair +-v is shared; 106 operations a component where velocity by velocity
+// took 142).  J = j^s or rho^s u (Eq. ff3).  w_i rho^s/tau enters last, so that it is not rounded
+// together with the velocity terms.
+template <typename C>
+struct Collision19 {
+    C keep, k0, tr, hb, l[3], B[3], Bxy, Bxz, Byz, txy, txz, tyz;
+    __device__ __forceinline__ Collision19(const StepParams<C>& p, C r, const C (&j)[3], const C (&u)[3],
+                                           const C (&a)[3])
+    {
+        keep = C(1) - p.omega;
+        k0 = p.omega * r;
+        C o[3];
+#pragma unroll
+        for (int d = 0; d < 3; ++d) {
+            o[d] = k0 * u[d];
+            l[d] = fma(r, a[d], o[d]);
+            B[d] = fma(C(0.5) * o[d], u[d], a[d] * j[d]);
+        }
+        Bxy = fma(o[0], u[1], fma(a[0], j[1], a[1] * j[0]));
+        Bxz = fma(o[0], u[2], fma(a[0], j[2], a[2] * j[0]));
+        Byz = fma(o[1], u[2], fma(a[1], j[2], a[2] * j[1]));
+        tr = (B[0] + B[1]) + B[2];
+        const C b = C(-1.0 / 3.0) * tr, qb = C(0.25) * b;
+        hb = C(0.5) * b;
+        txy = fma(C(0.25), B[0] + B[1], qb);
+        txz = fma(C(0.25), B[0] + B[2], qb);
+        tyz = fma(C(0.25), B[1] + B[2], qb);
+    }
+    // rest population; pair k = 1..9: velocities 2k - 1 and 2k
+    __device__ __forceinline__ C rest(C f) const { return fma(keep, f, fma(w19<C>(0), k0, -tr)); }
+    __device__ __forceinline__ void pair(int k, C f0, C f1, C& out0, C& out1) const
+    {
+        C even, odd, w;
+        if (k <= 3) {
+            even = fma(C(0.5), B[k - 1], hb);
+            odd = l[k - 1];
+            w = C(1.0 / 6.0);
+        } else {
+            const int q = (k - 4) >> 1;   // xy, xz, yz
+            const bool minus = (k & 1) != 0;
+            const C t = q == 0 ? txy : q == 1 ? txz : tyz, m = q == 0 ? Bxy : q == 1 ? Bxz : Byz;
+            const C la = q == 2 ? l[1] : l[0], lb = q == 0 ? l[1] : l[2];
+            even = fma(minus ? C(-0.25) : C(0.25), m, t);
+            odd = minus ? la - lb : la + lb;
+            w = C(1.0 / 12.0);
+        }
+        const C wk = w19<C>(2 * k);
+        out0 = fma(keep, f0, fma(wk, k0, fma(w, odd, even)));
+        out1 = fma(keep, f1, fma(wk, k0, fma(-w, odd, even)));
+    }
+};
+
+// rho^s and what is given of: js, the momenta j^s = sum_i f^s_i v_i ([s][d][site]) that the
+// collision would otherwise pull the populations a second time to form; total, the total momentum
+// ([d][site], stashed in the output U).  (An instance without the momenta was the slower one for
+// the march's step too: 192^3 x 3 903 us a step against 895, 200 x 180 x 190 x 2 647 against 642.)
 template <typename T, int N>
 __global__ void __launch_bounds__(SITE_THREADS)
 k19_density(const T* __restrict__ f, typename Storage<T>::C* __restrict__ rs,
@@ -160,10 +273,12 @@ k19_density(const T* __restrict__ f, typename Storage<T>::C* __restrict__ rs,
 {
     using C = typename Storage<T>::C;
     const long long site = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    grid_dependency_wait();
+    grid_dependents_launch();
     if (site >= p.S) return;
     const Site3 c = site3(p, site);
     const Hood3 h = hood3(p, c);
-    C r[N], j[N][3];
+    C r[N], j[N][3], held[N];
 #pragma unroll
     for (int s = 0; s < N; ++s) r[s] = j[s][0] = j[s][1] = j[s][2] = C(0);
 #pragma unroll
@@ -173,9 +288,7 @@ k19_density(const T* __restrict__ f, typename Storage<T>::C* __restrict__ rs,
         for (int s = 0; s < N; ++s) {
             const C v = Storage<T>::load(src + (long long)s * Q19 * p.S);
             r[s] += v;
-#pragma unroll
-            for (int d = 0; d < 3; ++d)
-                if (c19(i, d)) j[s][d] += C(c19(i, d)) * v;
+            momentum19(i, v, held[s], j[s]);
         }
     }
 #pragma unroll
@@ -201,18 +314,16 @@ template <typename C, int N>
 __device__ __forceinline__ void laplacians19(const C* __restrict__ rs, const StepParams<C>& p,
                                              const Site3& c, const C (&r)[N], C (&lap)[N])
 {
-    C acc[N];
     const Hood3 h = hood3(p, c);
-#pragma unroll
-    for (int s = 0; s < N; ++s) acc[s] = C(0);
+    C g[N][Q19];
 #pragma unroll
     for (int i = 1; i < Q19; ++i) {
         const long long t = fnb3(p, c, h, i);
 #pragma unroll
-        for (int s = 0; s < N; ++s) acc[s] += w19<C>(i) * (rs[s * p.S + t] - r[s]);
+        for (int s = 0; s < N; ++s) g[s][i] = rs[s * p.S + t];
     }
 #pragma unroll
-    for (int s = 0; s < N; ++s) lap[s] = C(6) * acc[s];
+    for (int s = 0; s < N; ++s) lap[s] = lap19(r[s], [&](int i) { return g[s][i]; });
 }
 
 template <typename C, int N>
@@ -220,6 +331,8 @@ __global__ void __launch_bounds__(SITE_THREADS)
 k19_potential(const C* __restrict__ rs, C* __restrict__ nu, const __grid_constant__ StepParams<C> p)
 {
     const long long site = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    grid_dependency_wait();
+    grid_dependents_launch();
     if (site >= p.S) return;
     const Site3 c = site3(p, site);
     C r[N], lap[N], out[N];
@@ -255,23 +368,15 @@ __device__ __forceinline__ void grads19(const C* __restrict__ g, const StepParam
                                         const Site3& c, C (&gr)[N][3])
 {
     const Hood3 h = hood3(p, c);
-#pragma unroll
-    for (int s = 0; s < N; ++s) gr[s][0] = gr[s][1] = gr[s][2] = C(0);
+    C v[N][Q19];
 #pragma unroll
     for (int i = 1; i < Q19; ++i) {
         const long long t = fnb3(p, c, h, i);
 #pragma unroll
-        for (int s = 0; s < N; ++s) {
-            const C v = w19<C>(i) * g[s * p.S + t];
-#pragma unroll
-            for (int d = 0; d < 3; ++d)
-                if (c19(i, d)) gr[s][d] += C(c19(i, d)) * v;
-        }
+        for (int s = 0; s < N; ++s) v[s][i] = g[s * p.S + t];
     }
 #pragma unroll
-    for (int s = 0; s < N; ++s)
-#pragma unroll
-        for (int d = 0; d < 3; ++d) gr[s][d] *= C(3);
+    for (int s = 0; s < N; ++s) gradient19<C>([&](int i) { return v[s][i]; }, gr[s]);
 }
 
 // Accelerations a^s (Eq. definef plus the body force; with p.gd the Gibbs-Duhem shift
@@ -287,7 +392,7 @@ __device__ __forceinline__ void accel19(const C* __restrict__ rs, const C* __res
 #pragma unroll
     for (int s = 0; s < N; ++s)
 #pragma unroll
-        for (int d = 0; d < 3; ++d) a[s][d] = -p.fcoef * a[s][d] + g[d];
+        for (int d = 0; d < 3; ++d) a[s][d] = fma(-p.fcoef, a[s][d], g[d]);
     if (p.gd) {
         C grt[3] = {C(0), C(0), C(0)};
         C gs[N][3];
@@ -320,6 +425,8 @@ k19_collide(const T* __restrict__ fin, T* __restrict__ fout,
 {
     using C = typename Storage<T>::C;
     const long long site = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    grid_dependency_wait();
+    grid_dependents_launch();
     if (site >= p.S) return;
     const Site3 c = site3(p, site);
     const Hood3 h = hood3(p, c);
@@ -340,46 +447,26 @@ k19_collide(const T* __restrict__ fin, T* __restrict__ fout,
     }
     const C inv = C(1) / rho;
     const C u[3] = {jt[0] * inv, jt[1] * inv, jt[2] * inv};
-    const C base = C(-1.5) * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
     C a[N][3];
     accel19<C, N>(rs, nu, p, c, r, rho, a);
-    // f* = f (1 - 1/tau) + (rho^s/tau) e_i + w_i [3 rho^s (v.a) + 9 (v.a)(v.J) - 3 a.J
-    // + rho^s/tau], e_i = w_i (3 v.u + 9/2 (v.u)^2 - 3/2 u.u), J = j^s or rho^s u (Eq. ff3);
-    // J is kept in j, and the per-component constants are formed once
-    C r3[N], omr[N], m3aj[N];
+    const Nb3 here = nb3(p, c, 0, 0, 0);
+    T* dst = fout + at19(p, 0, here.row, here.x);
 #pragma unroll
     for (int s = 0; s < N; ++s) {
         if (p.bary)
 #pragma unroll
             for (int d = 0; d < 3; ++d) j[s][d] = r[s] * u[d];
-        r3[s] = C(3) * r[s];
-        omr[s] = p.omega * r[s];
-        m3aj[s] = fma(C(-3), a[s][0] * j[s][0] + a[s][1] * j[s][1] + a[s][2] * j[s][2], omr[s]);
-    }
-    const C keep = C(1) - p.omega;
-    const Nb3 here = nb3(p, c, 0, 0, 0);
-    T* dst = fout + at19(p, 0, here.row, here.x);
+        const Collision19<C> col(p, r[s], j[s], u, a[s]);
+        const T* src = fin + s * cstride;
+        T* out = dst + s * cstride;
+        out[0] = T(col.rest(Storage<T>::load(src + src19(p, c, h, 0))));
 #pragma unroll
-    for (int i = 0; i < Q19; ++i) {
-        C cu = C(0);
-#pragma unroll
-        for (int d = 0; d < 3; ++d)
-            if (c19(i, d)) cu += C(c19(i, d)) * u[d];
-        const C e = (i == 0) ? w19<C>(0) * base : w19<C>(i) * fma(cu, fma(C(4.5), cu, C(3)), base);
-        const T* src = fin + src19(p, c, h, i);
-#pragma unroll
-        for (int s = 0; s < N; ++s) {
-            C ca = C(0), cj = C(0);
-#pragma unroll
-            for (int d = 0; d < 3; ++d)
-                if (c19(i, d)) {
-                    ca += C(c19(i, d)) * a[s][d];
-                    cj += C(c19(i, d)) * j[s][d];
-                }
-            const C F = (i == 0) ? w19<C>(0) * m3aj[s]
-                                 : w19<C>(i) * fma(ca, fma(C(9), cj, r3[s]), m3aj[s]);
-            const C v = Storage<T>::load(src + s * cstride);
-            dst[s * cstride + (long long)i * p.nx] = T(fma(keep, v, fma(omr[s], e, F)));
+        for (int k = 1; k <= 9; ++k) {
+            C o0, o1;
+            col.pair(k, Storage<T>::load(src + src19(p, c, h, 2 * k - 1)),
+                     Storage<T>::load(src + src19(p, c, h, 2 * k)), o0, o1);
+            out[(long long)(2 * k - 1) * p.nx] = T(o0);
+            out[(long long)(2 * k) * p.nx] = T(o1);
         }
     }
     if (!(rho > C(0)) || !isfinite(rho)) atomicOr(p.status, STATUS_NONFINITE);
@@ -453,7 +540,7 @@ k19_set_state(const double* __restrict__ in, T* __restrict__ f,
 // = u + (sum_s rho^s a^s)/(2 rho) (Eq. scon); mu^s; P (6 * S: xx, xy, xz, yy, yz, zz) =
 // (sum_s rho^s mu^s - psi) I + kappa sum_s grad rho^s grad rho^s (Eq. ppp, diagnostic).
 template <typename C, int N>
-__global__ void __launch_bounds__(SITE_THREADS)
+__global__ void __launch_bounds__(SITE_THREADS, sizeof(C) == 4 && N <= 4 ? 4 : 1)
 k19_moments(const C* __restrict__ rs, const C* __restrict__ nu, double* __restrict__ rho_out,
             double* __restrict__ U, double* __restrict__ mu_out, double* __restrict__ P,
             const __grid_constant__ StepParams<C> p)

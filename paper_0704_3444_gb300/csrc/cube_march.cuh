@@ -144,6 +144,8 @@ k19_march(const T* __restrict__ fin, T* __restrict__ fout,
     constexpr int NA = (M3_ROWS + M3_WARPS - 1) / M3_WARPS;
     const bool xout = lane >= 2 && lane < 30 && x0 + lane - 2 < nx;
 
+    grid_dependency_wait();
+    grid_dependents_launch();
     const int nk = Hc + 4;
     for (int k = 0; k < nk; ++k) {
         const int m = z0 - 2 + k;
@@ -172,22 +174,14 @@ k19_march(const T* __restrict__ fin, T* __restrict__ fout,
             for (int j = 0; j < NA; ++j) {
                 const int r = warp + M3_WARPS * j;
                 if (r >= 1 && r < M3_ROWS - 1) {
-                    C rr[N], acc[N], lap[N], out[N];
+                    C rr[N], lap[N], out[N];
 #pragma unroll
                     for (int s = 0; s < N; ++s) {
                         rr[s] = rring[m3_at<N>(qc, s, r, lane)];
-                        acc[s] = C(0);
+                        lap[s] = lap19(rr[s], [&](int i) {
+                            return rring[m3_at<N>(qz[1 + c19(i, 2)], s, r + c19(i, 1), lane + c19(i, 0))];
+                        });
                     }
-#pragma unroll
-                    for (int i = 1; i < Q19; ++i) {
-                        const int q = qz[1 + c19(i, 2)];
-                        const int rn = r + c19(i, 1), ln = lane + c19(i, 0);
-#pragma unroll
-                        for (int s = 0; s < N; ++s)
-                            acc[s] += w19<C>(i) * (rring[m3_at<N>(q, s, rn, ln)] - rr[s]);
-                    }
-#pragma unroll
-                    for (int s = 0; s < N; ++s) lap[s] = C(6) * acc[s];
                     site_nu<C, N>(p, rr, lap, out);
 #pragma unroll
                     for (int s = 0; s < N; ++s) nring[m3_at<N>(k % 3, s, r, lane)] = out[s];
@@ -211,16 +205,13 @@ k19_march(const T* __restrict__ fin, T* __restrict__ fout,
                 m3_pull<T, N>(fin, cst, xw, rw, zz, ny, nx, v);
                 C rs[N], js[N][3];
 #pragma unroll
-                for (int s = 0; s < N; ++s) rs[s] = js[s][0] = js[s][1] = js[s][2] = C(0);
+                for (int s = 0; s < N; ++s) {
+                    rs[s] = v[s][0];
 #pragma unroll
-                for (int i = 0; i < Q19; ++i)
+                    for (int i = 1; i < Q19; ++i) rs[s] += v[s][i];
 #pragma unroll
-                    for (int s = 0; s < N; ++s) {
-                        rs[s] += v[s][i];
-#pragma unroll
-                        for (int d = 0; d < 3; ++d)
-                            if (c19(i, d)) js[s][d] += C(c19(i, d)) * v[s][i];
-                    }
+                    for (int q = 1; q <= 9; ++q) add_momentum19(q, v[s][2 * q - 1] - v[s][2 * q], js[s]);
+                }
                 C rho = C(0), jt[3] = {C(0), C(0), C(0)};
 #pragma unroll
                 for (int s = 0; s < N; ++s) {
@@ -230,64 +221,29 @@ k19_march(const T* __restrict__ fin, T* __restrict__ fout,
                 }
                 const C inv = C(1) / rho;
                 const C u[3] = {jt[0] * inv, jt[1] * inv, jt[2] * inv};
-                const C base = C(-1.5) * (u[0] * u[0] + u[1] * u[1] + u[2] * u[2]);
-                // a^s = -(1 - 1/2tau) grad nu^s + g, grad g = 3 sum_i w_i v_i g(r + v_i)
-                C a[N][3];
-#pragma unroll
-                for (int s = 0; s < N; ++s) a[s][0] = a[s][1] = a[s][2] = C(0);
-#pragma unroll
-                for (int i = 1; i < Q19; ++i) {
-                    const int q = qn[1 + c19(i, 2)];
-                    const int rn = r + c19(i, 1), ln = lane + c19(i, 0);
-#pragma unroll
-                    for (int s = 0; s < N; ++s) {
-                        const C g = w19<C>(i) * nring[m3_at<N>(q, s, rn, ln)];
-#pragma unroll
-                        for (int d = 0; d < 3; ++d)
-                            if (c19(i, d)) a[s][d] += C(c19(i, d)) * g;
-                    }
-                }
+                // a^s = -(1 - 1/2tau) grad nu^s + g, then the collision
                 const C gb[3] = {p.gx, p.gy, p.gz};
-#pragma unroll
-                for (int s = 0; s < N; ++s)
-#pragma unroll
-                    for (int d = 0; d < 3; ++d) a[s][d] = -p.fcoef * (C(3) * a[s][d]) + gb[d];
-                // f* = f (1 - 1/tau) + (rho^s/tau) e_i + w_i [3 rho^s (v.a) + 9 (v.a)(v.J)
-                // - 3 a.J + rho^s/tau] (as in k19_collide)
-                C r3[N], omr[N], m3aj[N];
+                const unsigned here = m3_rowbase(zz[1], rw.y[1], ny, nx) + (unsigned)xw[1];
 #pragma unroll
                 for (int s = 0; s < N; ++s) {
+                    C a[3];
+                    gradient19<C>([&](int i) {
+                        return nring[m3_at<N>(qn[1 + c19(i, 2)], s, r + c19(i, 1), lane + c19(i, 0))];
+                    }, a);
+#pragma unroll
+                    for (int d = 0; d < 3; ++d) a[d] = fma(-p.fcoef, a[d], gb[d]);
                     if (p.bary)
 #pragma unroll
                         for (int d = 0; d < 3; ++d) js[s][d] = rs[s] * u[d];
-                    r3[s] = C(3) * rs[s];
-                    omr[s] = p.omega * rs[s];
-                    m3aj[s] = fma(C(-3), a[s][0] * js[s][0] + a[s][1] * js[s][1] + a[s][2] * js[s][2],
-                                  omr[s]);
-                }
-                const C keep = C(1) - p.omega;
-                const unsigned here = m3_rowbase(zz[1], rw.y[1], ny, nx) + (unsigned)xw[1];
+                    const Collision19<C> col(p, rs[s], js[s], u, a);
+                    T* out = fout + (size_t)s * cst;
+                    out[here] = T(col.rest(v[s][0]));
 #pragma unroll
-                for (int i = 0; i < Q19; ++i) {
-                    C cu = C(0);
-#pragma unroll
-                    for (int d = 0; d < 3; ++d)
-                        if (c19(i, d)) cu += C(c19(i, d)) * u[d];
-                    const C e = (i == 0) ? w19<C>(0) * base
-                                         : w19<C>(i) * fma(cu, fma(C(4.5), cu, C(3)), base);
-#pragma unroll
-                    for (int s = 0; s < N; ++s) {
-                        C ca = C(0), cj = C(0);
-#pragma unroll
-                        for (int d = 0; d < 3; ++d)
-                            if (c19(i, d)) {
-                                ca += C(c19(i, d)) * a[s][d];
-                                cj += C(c19(i, d)) * js[s][d];
-                            }
-                        const C F = (i == 0) ? w19<C>(0) * m3aj[s]
-                                             : w19<C>(i) * fma(ca, fma(C(9), cj, r3[s]), m3aj[s]);
-                        fout[(size_t)s * cst + here + (unsigned)(i * nx)] =
-                            T(fma(keep, v[s][i], fma(omr[s], e, F)));
+                    for (int k = 1; k <= 9; ++k) {
+                        C o0, o1;
+                        col.pair(k, v[s][2 * k - 1], v[s][2 * k], o0, o1);
+                        out[here + (unsigned)((2 * k - 1) * nx)] = T(o0);
+                        out[here + (unsigned)(2 * k * nx)] = T(o1);
                     }
                 }
                 if (!(rho > C(0)) || !isfinite(rho)) atomicOr(p.status, STATUS_NONFINITE);

@@ -104,6 +104,7 @@ struct LatticeTable {
     // set up the single-pass step where it applies (P.seg3, P.grid3): 1 = set up, 0 = the
     // staged step, -1 = CUDA error; null for lattices with one step kernel
     int (*plan)(Problem& P, int sm_count);
+    bool (*pays)(const Problem& P);   // whether AUTO should take that step (null: always)
     size_t item_bytes;            // size of the device description at Scratch::line_item
     // write the description of buffers f[0], f[1] to sc.line_item (synchronous)
     cudaError_t (*prepare)(const Problem&, const Scratch&, void* const* f);

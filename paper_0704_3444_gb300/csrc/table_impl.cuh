@@ -783,6 +783,13 @@ struct Launch19 {
             return 1;
         }
     }
+    // The march pays up to three components from about 1e6 site-components on (us per step, march
+    // / staged: 192^3 x 3 895 / 1056, 100 x 90 x 70 x 2 66 / 73, 128 x 120 x 100 x 4 311 / 311; 64 x
+    // 60 x 50 x 3 50 / 28, 40 x 24 x 30 x 3 37 / 10: too few CTAs, each with its dependent plane
+    // iterations), and not in FP64, which the FP64 pipe bounds and whose pulled values spill
+    // (64^3 x 3 877 / 355, 128 x 128 x 96 x 2 2477 / 1396).
+    static bool pays(const Problem& P) { return sizeof(C) == 4 && P.N <= 3 && P.S * P.N >= 1200000; }
+
     static int plan(Problem& P, int sm_count)
     {
         switch (P.N) {
@@ -822,26 +829,42 @@ struct Launch19 {
             if constexpr (NN <= M3_NMAX) {
                 if (P.seg3 > 0) {
                     const dim3 grid(P.grid3[0], P.grid3[1], P.grid3[2]);
+                    // dependent launches hide the launch, but the CTAs that come early crowd the
+                    // last wave (100 x 90 x 70 x 2 75 -> 70 us, 192^3 x 3 923 -> 941)
+                    const bool dependent = P.S * P.N < 6000000;
                     for (; nsteps > 0; --nsteps) {
                         const T* fi = (const T*)f[*cur];
-                        k19_density<T, NN><<<site_blocks(P.S), SITE_THREADS, 0, st>>>(
-                            fi, (C*)sc.rho_s, nullptr, p);
-                        k19_march<T, NN><<<grid, M3_THREADS, m3_smem_bytes<C, NN>(), st>>>(
-                            fi, (T*)f[*cur ^ 1], (const C*)sc.rho_s, p, P.seg3);
-                        const cudaError_t e = cudaGetLastError();
+                        cudaError_t e;
+                        if (dependent) {
+                            e = launch_dependent(k19_density<T, NN>, dim3(site_blocks(P.S)), SITE_THREADS,
+                                                 0, st, fi, (C*)sc.rho_s, nullptr, p, nullptr);
+                            if (e == cudaSuccess)
+                                e = launch_dependent(k19_march<T, NN>, grid, M3_THREADS, m3_smem_bytes<C, NN>(),
+                                                     st, fi, (T*)f[*cur ^ 1], (const C*)sc.rho_s, p, P.seg3);
+                        } else {
+                            k19_density<T, NN><<<site_blocks(P.S), SITE_THREADS, 0, st>>>(
+                                fi, (C*)sc.rho_s, nullptr, p);
+                            k19_march<T, NN><<<grid, M3_THREADS, m3_smem_bytes<C, NN>(), st>>>(
+                                fi, (T*)f[*cur ^ 1], (const C*)sc.rho_s, p, P.seg3);
+                            e = cudaGetLastError();
+                        }
                         if (e != cudaSuccess) return e;
                         *cur ^= 1;
                     }
                     return cudaSuccess;
                 }
             }
+            // the staged step; few sites: smaller blocks, so that every SM has one
+            const int th = P.S < 4LL * 152 * SITE_THREADS ? 64 : SITE_THREADS;
+            const dim3 grid((unsigned)((P.S + th - 1) / th));
             for (; nsteps > 0; --nsteps) {
-                cudaError_t e = fields_n<NN>(p, sc, (const T*)f[*cur], st);
-                if (e != cudaSuccess) return e;
-                k19_collide<T, NN><<<site_blocks(P.S), SITE_THREADS, 0, st>>>(
-                    (const T*)f[*cur], (T*)f[*cur ^ 1], (const C*)sc.rho_s, (const C*)sc.js,
-                    (const C*)sc.nu, p);
-                e = cudaGetLastError();
+                cudaError_t e = launch_dependent(k19_density<T, NN>, grid, th, 0, st, (const T*)f[*cur],
+                                                 (C*)sc.rho_s, (C*)sc.js, p, nullptr);
+                if (e == cudaSuccess)
+                    e = launch_dependent(k19_potential<C, NN>, grid, th, 0, st, (const C*)sc.rho_s, (C*)sc.nu, p);
+                if (e == cudaSuccess)
+                    e = launch_dependent(k19_collide<T, NN>, grid, th, 0, st, (const T*)f[*cur],
+                                         (T*)f[*cur ^ 1], (const C*)sc.rho_s, (const C*)sc.js, (const C*)sc.nu, p);
                 if (e != cudaSuccess) return e;
                 *cur ^= 1;
             }
@@ -855,7 +878,7 @@ struct Launch19 {
         const auto p = make_params<C>(P, sc.status);
         MCLB_DISPATCH_N(P.N, {
             k19_density<T, NN><<<site_blocks(P.S), SITE_THREADS, 0, st>>>((const T*)f, (C*)sc.rho_s,
-                                                                          nullptr, p, U);
+                                                                                nullptr, p, U);
             if (U)
                 k19_potential<C, NN><<<site_blocks(P.S), SITE_THREADS, 0, st>>>((const C*)sc.rho_s,
                                                                                 (C*)sc.nu, p);
@@ -919,6 +942,7 @@ struct Launch19 {
             LatticeTable x{};
             x.max_resident = &max_resident;
             x.plan = &plan;
+            x.pays = &pays;
             x.item_bytes = 0;
             x.prepare = &prepare;
             x.init = &init;

@@ -234,3 +234,29 @@ def test_fit_equilibrium_on_slabs():
     assert np.max(np.abs(fit - want)) < 1e-12
     assert np.max(np.abs(fit[0] - hi)) < 0.05 and np.max(np.abs(fit[1] - lo)) < 0.05
     sim.close()
+
+
+@pytest.mark.parametrize("n,shape,precision", [(3, (19, 7, 5), "fp64"), (1, (3, 2, 1), "fp64"), (4, (40, 30, 17), "fp32"),
+                                               (3, (96, 90, 52), "fp32")], ids=str)
+def test_auto_schedule(n, shape, precision):
+    """What AUTO takes -- the staged step in FP64, for small lattices and from four components
+    on, the march above -- against the oracle after 12 steps with every term on."""
+    nx, ny, nz = shape
+    rng = np.random.default_rng(41 + nx)
+    rho = (1.0 + 0.1 * rng.uniform(-1, 1, (n, nz, ny, nx))) / n
+    u = 0.03 * rng.uniform(-1, 1, (3, nz, ny, nx))
+    kw = dict(m=[1.0 + (k % 3) for k in range(n)], theta=0.4, kappa=0.02, force=(1e-5, -2e-5, 3e-5),
+              forcing_velocity=n % 2, lattice="d3q19", nz=nz)
+    chi = inputs.uniform_chi(n, 1.6)
+    sim = mclb.Simulation(n, nx, ny, 0.9, chi, precision=precision, **kw)
+    assert sim.launches_per_step == (2 if n * nx * ny * nz > 1200000 else 3)
+    orc = Oracle(n, nx, ny, 0.9, chi, **kw)
+    sim.init_fields(rho, u)
+    orc.init(rho, u)
+    sim.step(12)
+    assert orc.run(12) == 0
+    assert sim.status() == 0
+    gm, om = sim.moments(), orc.moments()
+    for k in ("rho", "U", "mu"):
+        assert np.max(np.abs(gm[k] - om[k])) < (1e-12 if precision == "fp64" else 1e-5), k
+    sim.close()
