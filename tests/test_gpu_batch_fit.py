@@ -321,6 +321,26 @@ def test_fit_equilibrium_matches_its_definition(nphase):
     sim.close()
 
 
+@pytest.mark.parametrize("nphase", [2, 3])
+@pytest.mark.parametrize("nx,ny", [(13, 9), (48, 40), (256, 192)])
+def test_fit_equilibrium_over_many_iterations(nx, ny, nphase):
+    """Smooth fields without phases, which take k-means 4 to 20 iterations (within, exactly at
+    and past the device's run of 10), against the same fit in numpy.  No site lies nearer than
+    9e-10 to a tie of two centroids, so both take the same path; a mean of 49152 values near
+    1/3, added in either order, is good to 1e-12."""
+    y, x = np.mgrid[0:ny, 0:nx]
+    X, Y, a = 2 * np.pi * x / nx, 2 * np.pi * y / ny, 3e-3 * min(nx, ny) / 48
+    rho = np.stack([1 + a * (np.sin(X) + 0.6 * np.cos(2 * X + Y) + 0.3 * np.sin(Y)),
+                    1 + a * (np.cos(X + Y) + 0.5 * np.sin(Y)),
+                    1 + a * 0.4 * np.cos(2 * Y)])
+    sim = mclb.Simulation(3, nx, ny, 0.9, inputs.uniform_chi(3, 1.0), precision="fp64")
+    sim.init_fields(rho)
+    got = sim.fit_equilibrium(nphase)
+    want = _fit_by_definition(sim.moments(U=False, mu=False, P=False)["rho"], nphase)
+    np.testing.assert_allclose(got, want, rtol=0, atol=1e-12)
+    sim.close()
+
+
 @pytest.mark.parametrize("precision", ["fp32", "bf16"])
 def test_every_autotuner_candidate_matches_single_handles(precision):
     """The autotuner times every partition (wide and narrow strips, segment heights for 2,
