@@ -243,22 +243,46 @@ std::vector<MarchCta> march_ctas(int count, const Problem* probs, int slots, int
 }
 
 // Whether a group's instances step by tiles instead of the march.
-//   FP32: row tiles where every instance has rows enough and the group keeps the GPU busy (48
-//     instances of 32^2 to 512^2, N = 2 and 3: 153 us a step, 184 by the march with its ghost
-//     launch; 300 of 32^2 to 200^2: 231 / 307), up to the five components whose CTAs share an SM.
+//   FP32, groups that keep the GPU busy (1e6 site-components) of instances with rows enough: row
+//     tiles run at 27k (64^2) to 58k (1000^2) site-components a us whatever the number of instances, the
+//     march with its ghost launch at 18k to 71k: it wants instances that fill its strips and segments,
+//     and more of them the fewer components there are.  us a step, tiles / march, instances of
+//     s x s and site-components in all:
+//       N = 1: 512^2 16e6 289 / 351, 48e6 848 / 974: always
+//       N = 2: 64^2 4e6 125 / 186, 250^2 48e6 926 / 1005, 400^2 4e6 80.0 / 80.9, 16e6 304 / 288; sizes
+//         32 to 512 41e6 824 / 827, 200 to 512 26e6 494 / 469: below 255^2 on average, or few sites
+//       N = 3: 64^2 4e6 124 / 173, 150^2 16e6 366 / 418, 250^2 4e6 86 / 95, 16e6 317 / 304, 512^2 48e6
+//         886 / 737, 1000^2 3e6 61.8 / 57.6; sizes 32 to 200 11e6 274 / 318, 32 to 512 5.2e6 112 / 120,
+//         32e6 647 / 601: below 200^2, or 390^2 and few (but 100^2, which the strips just hold, 1e6
+//         32.8 / 29.5).  Beside another group the tiles' even CTAs count for more: 20 of sizes 200 to
+//         512, N = 2 and 3, 119 by tiles, 137 with N = 3 by the march
+//       N = 4: 64^2 4e6 131 / 175, 150^2 4e6 103 / 111, 250^2 4e6 92 / 91
+//       N = 5: 64^2 1e6 36.6 / 48.1, 100^2 1e6 33.3 / 30.2, 2e6 62.5 / 61.5, 4e6 114 / 122, 150^2 4e6
+//         103 / 114, 250^2 16e6 339 / 318, 512^2 16e6 321 / 241
 //   FP64: the tiles spend fewer FP64 instructions than the march (table_impl.cuh has both sides),
 //     but for four and five components.
 template <typename T>
 bool batch_takes_tiles(int N, int count, const Problem* probs)
 {
-    long long work = 0;
+    long long sites = 0;
     int rows = INT32_MAX;
     for (int k = 0; k < count; ++k) {
-        work += probs[k].S * N;
+        sites += probs[k].S;
         rows = std::min(rows, probs[k].ny);
         if ((long long)probs[k].plane * N >= (1LL << 31)) return false;
     }
-    if (std::is_same<T, float>::value) return N <= ROWS_NMAX && rows >= ROWS_MIN_NY && work >= 1000000;
+    if (std::is_same<T, float>::value) {
+        const long long work = sites * N, mean = sites / count;
+        if (rows < ROWS_MIN_NY || work < 1000000) return false;
+        switch (N) {
+            case 1: return true;
+            case 2: return mean < 65000 || work < 5000000;
+            case 3: return mean < 40000 || (mean < 150000 && work < 6000000);
+            case 4:
+            case 5: return mean < 8000 || (mean < 30000 && work >= 2000000);
+            default: return false;   // (more do not share an SM: ROWS_NMAX)
+        }
+    }
     if (std::is_same<T, double>::value) return N != 4 && N != 5;
     return false;
 }

@@ -1079,14 +1079,25 @@ cudaError_t batch_fork(mclb_batch b)
     return e == cudaSuccess ? cudaStreamWaitEvent(b->side, b->ev_fork, 0) : e;
 }
 
+// Whether the groups' launches share SMs: all by tiles or none.  (Tiles and the march divide an SM's
+// memory differently, and it changes over only when idle: 512 instances of 32^2 to 512^2 with N = 2
+// by tiles beside N = 3 by the march ran at 47.0k MLUPS x N, both by the march at 54.6k.)
+bool batch_alike(mclb_batch b)
+{
+    size_t tiles = 0;
+    for (const void* g : b->groups) tiles += b->tab->batch_waves(g) % 1000 == 1 ? 1 : 0;
+    return tiles == 0 || tiles == b->groups.size();
+}
+
 // One batched timestep.  A group depends on nothing but its own last step, so every second group
 // runs its chain of launches on the side stream, beside the others: each fills the SMs that
 // the other's last wave leaves idle (48 instances of N = 2 and 3, FP32 by tiles: 176 us a step
 // one after the other, 153 side by side).
 cudaError_t batch_launch(mclb_batch b, int parity)
 {
+    const bool beside = batch_alike(b);
     for (size_t g = 0; g < b->groups.size(); ++g) {
-        cudaStream_t st = (g & 1) ? b->side : b->stream;
+        cudaStream_t st = (g & 1) && beside ? b->side : b->stream;
         cudaError_t e = b->tab->batch_step(b->groups[g], parity, st, 0);
         if (e == cudaSuccess) e = b->tab->batch_step(b->groups[g], parity, st, 1);
         if (e == cudaSuccess) e = cudaEventRecord(b->ev_side[g], st);

@@ -178,3 +178,27 @@ def test_march_between_walls_with_wall_tiles(precision, shape, steps):
     if precision == "fp64":
         assert _rel(sim.get_state(), orc.f) < 1e-12
     sim.close()
+
+
+def test_fp32_batch_of_tiles_and_march():
+    """One group by row tiles and one, of few large instances, by the march: one after the other on
+    one stream, densities and U within the FP32 tolerance of the oracle (1e-5) after 35 steps (a
+    replayed graph and single steps)."""
+    probs = []
+    for k, (nx, ny, n) in enumerate([(700, 720, 2), (400, 423, 3), (409, 420, 3)]):
+        rho, u = inputs.random_state(n, nx, ny, seed=660 + k, amp=0.1, umax=0.03)
+        probs.append(inputs.Problem(name=f"m{k}", ncomp=n, nx=nx, ny=ny, tau=0.8 + 0.1 * k, chi=inputs.uniform_chi(n, 1.7),
+                                    m=np.ones(n), theta=1 / 3, kappa=0.01, force=(1e-5, 0.0), rho=rho, u=u))
+    b = mclb.Batch(probs, precision="fp32")
+    b.init_all()
+    b.step(35)
+    waves = [w for _, w in b.tuning()]
+    assert waves[0] == 1 and waves[1] in (2, 4, 8, 16) and b.launches_per_step == 3
+    assert b.status()[0] == 0
+    for k, p in enumerate(probs):
+        orc = Oracle.from_problem(p)
+        orc.run(35)
+        got, want = b.moments(k), orc.moments()
+        for f in ("rho", "U"):
+            assert np.max(np.abs(got[f] - want[f])) < 1e-5, (k, f)
+    b.close()
