@@ -536,7 +536,8 @@ k19_set_state(const double* __restrict__ in, T* __restrict__ f,
     }
 }
 
-// Output fields (after k19_density and k19_potential of the same state): rho^s; U (3 * S)
+// Output fields (after k19_density, which leaves the total momentum in U, and k19_potential of the
+// same state): rho^s; U (3 * S)
 // = u + (sum_s rho^s a^s)/(2 rho) (Eq. scon); mu^s; P (6 * S: xx, xy, xz, yy, yz, zz) =
 // (sum_s rho^s mu^s - psi) I + kappa sum_s grad rho^s grad rho^s (Eq. ppp, diagnostic).
 template <typename C, int N>

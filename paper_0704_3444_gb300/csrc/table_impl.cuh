@@ -2,6 +2,7 @@
 #pragma once
 
 #include <algorithm>
+#include <cmath>
 
 #include "batch.cuh"
 #include "cube.cuh"
@@ -740,12 +741,14 @@ struct Launch19 {
     static cudaError_t prepare(const Problem&, const Scratch&, void* const*) { return cudaSuccess; }
 
     // The march (cube_march.cuh) after a density pass: tiles of M3_OUT_X x M3_OUT_Y, z
-    // segments of H planes.  The CTAs are latency bound, so more of them than one wave
-    // of resident slots helps; a segment of H planes costs about H + 4 plane iterations (four
-    // warm-up planes) and the launch about waves x (H + 4) of them, so the segment count
-    // that minimises that product is taken.  Not for N > M3_NMAX, the Gibbs-Duhem reading
-    // (it needs grad rho on the density planes the next iteration overwrites) or
-    // 19 S >= 2^31 (32-bit offsets).
+    // segments of H planes.  The four warm-up planes of a segment collide nothing and cost about
+    // two; w waves of resident CTAs, which do not run in step, end about one CTA later and lose
+    // part of a last wave that is not full.  The segment count that minimises (w + 1 + 0.3 (ceil w
+    // - w)) (H + 2) is taken (us per step at 5 / 7 / 10 / 14 / 16 / 20 segments: 256^3 x 3 2351 / 2273 /
+    // 2168 / 2090 / 2095 / 2057; 192^3 x 3 938 / 902 / 873 / 855 / 867 / 887; 256 x 200 x 220 x 2 1124
+    // / 985 / 1031 / 979 / 996 / 1000; whole waves x (H + 4) took 7 in all three).  Not for N >
+    // M3_NMAX, the Gibbs-Duhem reading (it needs grad rho on the density planes the next
+    // iteration overwrites) or 19 S >= 2^31 (32-bit offsets).
     template <int N>
     static int plan_n(Problem& P, int sm_count)
     {
@@ -765,11 +768,11 @@ struct Launch19 {
             const long long tx = (P.nx + M3_OUT_X - 1) / M3_OUT_X, ty = (P.ny + M3_OUT_Y - 1) / M3_OUT_Y;
             const long long slots = (long long)ctas * std::max(1, sm_count);
             int best = 1;
-            long long best_cost = -1;
+            double best_cost = -1.0;
             for (int nseg = 1; nseg <= std::max(1, P.nz / 4); ++nseg) {
                 const long long H = (P.nz + nseg - 1) / nseg, segs = (P.nz + H - 1) / H;
-                const long long waves = (tx * ty * segs + slots - 1) / slots;
-                const long long cost = waves * (H + 4);
+                const double w = (double)(tx * ty * segs) / (double)slots;
+                const double cost = (w + 1.0 + 0.3 * (std::ceil(w) - w)) * (double)(H + 2);
                 if (best_cost < 0 || cost < best_cost) {
                     best_cost = cost;
                     best = nseg;
