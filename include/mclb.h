@@ -378,8 +378,9 @@ int mclb_step_noalloc(const mclb_params* params, const double* f_in, double* f_o
  * instance, column strip and row segment in a table built at the first step) and one
  * launch refreshes their ghost columns; where that kernel cannot be set up the group
  * falls back to the staged schedule (three launches).  Groups that small tiles step faster
- * (FP64; FP32 from about 1e6 site-components on) take those instead: one launch, two in
- * FP64.  Every second group's launches run beside the others'.  The first step after the batch
+ * (FP64; FP32 where at least 1e6 site-components are spread over few or small instances) take
+ * those instead: one launch, two in FP64.  Every second group's launches run beside the others',
+ * unless some groups take tiles and some do not.  The first step after the batch
  * is (re)built picks each march's work partition -- the strip shape (the single-lattice
  * kernel's, or a narrow one with two compute warps and 56 columns per CTA) and the segment
  * height (2, 4, 8 or 16 waves of resident CTAs) -- by timing every candidate on the current
