@@ -72,7 +72,9 @@ typedef enum {
 typedef enum {
     MCLB_KERNEL_AUTO = 0,   /* the fused single-pass kernel, or on lattices too small to
                                fill the GPU with it a kernel of small tiles (D2Q9, single
-                               handles): one launch per step, two with the Gibbs-Duhem form */
+                               handles): one launch per step, two with the Gibbs-Duhem form.
+                               In the 16-bit formats the state is that of FUSED bit for bit,
+                               whichever AUTO picks                                */
     MCLB_KERNEL_FUSED = 1,  /* stream, moments, potentials, force, collision in one
                                pass over the distributions, then a small launch that
                                refreshes the periodic ghost columns                 */
@@ -380,7 +382,9 @@ int mclb_step_noalloc(const mclb_params* params, const double* f_in, double* f_o
  * falls back to the staged schedule (three launches).  Groups that small tiles step faster
  * (FP64; FP32 where at least 1e6 site-components are spread over few or small instances) take
  * those instead: one launch, two in FP64.  Every second group's launches run beside the others',
- * unless some groups take tiles and some do not.  The first step after the batch
+ * unless some groups take tiles and some do not.  In the 16-bit formats with N >= 2 the batched march rounds
+ * one sum of nu^s where a handle's does not, so that an instance follows its own handle to the
+ * format's rounding, not bit for bit.  The first step after the batch
  * is (re)built picks each march's work partition -- the strip shape (the single-lattice
  * kernel's, or a narrow one with two compute warps and 56 columns per CTA) and the segment
  * height (2, 4, 8 or 16 waves of resident CTAs) -- by timing every candidate on the current

@@ -100,7 +100,7 @@ kb_march(const MarchItem<T>* __restrict__ items, const MarchCta* __restrict__ ct
                              : "memory");
     }
     __syncthreads();
-    march_cta<T, N, G>(&maps[parity][0], &maps[parity][1], &maps[parity ^ 1][2], &maps[parity ^ 1][3],
+    march_cta<T, N, G, false, true>(&maps[parity][0], &maps[parity][1], &maps[parity ^ 1][2], &maps[parity ^ 1][3],
                        it.f[parity ^ 1], ps, c.x0, c.y0, c.H, smem);
 }
 

@@ -292,7 +292,7 @@ __device__ __forceinline__ void store_site(T* f, const StepParams<C>& p, int s, 
         C dsum = C(0);
 #pragma unroll
         for (int i = 0; i < Q; ++i) {
-            const C d = Storage<T>::round(out[i] - wq<C>(i) * M);
+            const C d = Storage<T>::round(fma(-wq<C>(i), M, out[i]));
             dsum += d;
             store_row(f + line_off(p, s, y, i), x, p.nx, p.hx, d);
         }

@@ -134,7 +134,7 @@ constexpr bool has_narrow() { return MarchPick<T, N>::NW == 4 && MarchNarrow<T, 
 // The march of one CTA over the strip starting at column x0 and the segment of H rows
 // starting at row y0 (tmap/tmapr: load views of the input buffer; tmapw/tmapwr: store
 // views of fout; p may live in parameter or shared memory; G: the geometry).
-template <typename T, int N, typename G = MarchGeom<T, N>, bool GD = false>
+template <typename T, int N, typename G = MarchGeom<T, N>, bool GD = false, bool BATCH = false>
 __device__ __forceinline__ void march_cta(const CUtensorMap* tmap, const CUtensorMap* tmapr,
                                           const CUtensorMap* tmapw, const CUtensorMap* tmapwr,
                                           T* __restrict__ fout,
@@ -254,8 +254,8 @@ __device__ __forceinline__ void march_cta(const CUtensorMap* tmap, const CUtenso
 
     // FP32 storage collides two components at a time with the packed pair instructions
     constexpr bool PAIRS = std::is_same<T, float>::value && N >= 2;
-    const C theta = p.theta, kappa6 = C(6) * p.kappa;
-    const C c9 = C(1.0 / 9.0), c36 = C(1.0 / 36.0), c59 = C(5.0 / 9.0);
+    const C kappa6 = C(6) * p.kappa;
+    [[maybe_unused]] const C c9 = C(1.0 / 9.0), c36 = C(1.0 / 36.0);
 
     // The march over rows.  State carried from row to row
     // (m = lead row of the iteration about to start), per component:
@@ -317,18 +317,7 @@ __device__ __forceinline__ void march_cta(const CUtensorMap* tmap, const CUtenso
             if (out_lane && m >= ychk0 && m < ychk1 && (!(rho > C(0)) || !isfinite(rho)))
                 atomicOr(p.status, STATUS_NONFINITE);
             const C lnr = dev_log(rho);
-            C acc[N];
-            C sm = C(0), quad = C(0);
-#pragma unroll
-            for (int t = 0; t < N; ++t) {
-                C a = C(0);
-#pragma unroll
-                for (int u = 0; u < N; ++u) a += p.chi[t * N + u] * R0[u];
-                acc[t] = a;
-                sm += R0[t] * p.inv_m[t];
-                quad += R0[t] * a;
-            }
-            const C Gs = -theta * (sm * inv + C(0.5) * quad * inv * inv);
+            const SiteSums<C, N, (BATCH && N > 1)> sums(p, R0, inv);
             [[maybe_unused]] C Drn = C(0), Trn = C(0);
             if constexpr (GD) {
                 const C rl = __shfl_up_sync(0xffffffffu, rho, 1);
@@ -342,22 +331,16 @@ __device__ __forceinline__ void march_cta(const CUtensorMap* tmap, const CUtenso
 #pragma unroll
             for (int s = 0; s < N; ++s) {
                 const int c = s;
-                C logs = -p.th_m[s] * lnr;
-                if ((p.log_mask >> s) & 1u) {
-                    const C fl = p.log_floor * rho;
-                    logs += p.logc[s] * dev_log(R0[c] > fl ? R0[c] : fl);
-                }
-                const C L0 = logs + theta * (p.m_inv_m1[s] + acc[s] * inv) + Gs;
+                const C L0 = sums.nu(p, R0, rho, inv, lnr, s);
                 const C A = __shfl_up_sync(0xffffffffu, R0[c], 1) + __shfl_down_sync(0xffffffffu, R0[c], 1);
-                const C B0 = R0[c] * c9 + A * c36;
-                const C C0 = A * c9 - c59 * R0[c];
-                const C nu = Q1[c] - kappa6 * B0;
-                Q1[c] = Q0[c] + L0 - kappa6 * C0;
-                Q0[c] = -kappa6 * B0;
+                const C B0 = lap_side(R0[c], A);
+                const C nu = nu_whole(kappa6, Q1[c], B0);
+                Q1[c] = nu_part(kappa6, Q0[c], L0, lap_mid(R0[c], A));
+                Q0[c] = mul_rn(-kappa6, B0);
                 const C nl = __shfl_up_sync(0xffffffffu, nu, 1);
                 const C nr = __shfl_down_sync(0xffffffffu, nu, 1);
                 Dn[c] = nr - nl;
-                Tn[c] = nu * c9 + (nr + nl) * c36;
+                Tn[c] = grad_rows<N>(nu, nr + nl);
             }
 
             // ---- collision of row r = m - 2 (stage of iteration k - 2)
@@ -431,10 +414,8 @@ __device__ __forceinline__ void march_cta(const CUtensorMap* tmap, const CUtenso
                 };
                 // acceleration a^s of row r (Eq. definef plus the body force)
                 auto accel0 = [&](const int c, C& ax, C& ay) {
-                    const C gx = GX[c] + Dn[c] * c36;
-                    const C gy = Tn[c] - T2[c];
-                    ax = -p.fcoef * (C(3) * gx) + p.gx;
-                    ay = -p.fcoef * (C(3) * gy) + p.gy;
+                    ax = accel_of(p.fcoef, grad_cols(GX[c], Dn[c]), p.gx);
+                    ay = accel_of(p.fcoef, Tn[c] - T2[c], p.gy);
                 };
                 // GD: every component's a^s first, then the shift (A_c - A)/rho with A_c =
                 // (1 - 1/2tau) (1/3) grad rho from the total-density sums of rows r - 1 .. r + 1
@@ -510,7 +491,7 @@ __device__ __forceinline__ void march_cta(const CUtensorMap* tmap, const CUtenso
                     }
                 } else {
                     C e[Q];
-                    eq_weights(ux2, uy2, e);
+                    eq_weights(ux2, uy2, speed2(ux2, uy2), e);
 #pragma unroll
                     for (int c = 0; c < N; ++c) {
                         C f[Q], out[Q], ax, ay, fjx, fjy;
@@ -562,7 +543,7 @@ __device__ __forceinline__ void march_cta(const CUtensorMap* tmap, const CUtenso
             // ---- advance the carried state by one row
 #pragma unroll
             for (int c = 0; c < N; ++c) {
-                GX[c] = Dn[c] * c9 + Dp[c] * c36;
+                GX[c] = grad_cols_part(Dn[c], Dp[c]);
                 Dp[c] = Dn[c];
                 T2[c] = T1[c];
                 T1[c] = Tn[c];

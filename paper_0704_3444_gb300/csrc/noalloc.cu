@@ -113,7 +113,8 @@ k_na_collide(const double* __restrict__ fin, double* __restrict__ fout, const do
         jyt += by;
     }
     double e[Q];
-    eq_weights(jxt / rho, jyt / rho, e);
+    const double ux = jxt / rho, uy = jyt / rho;
+    eq_weights(ux, uy, fma(ux, ux, uy * uy), e);
 #pragma unroll
     for (int s = 0; s < N; ++s) {
         double gx, gy;

@@ -1,5 +1,10 @@
 // physics.cuh -- per-site arithmetic of one timestep (Li & Wagner, arXiv:0704.3444),
 // shared by the staged, fused and diagnostic kernels.
+//
+// Sums of products are written as explicit fused multiply-adds wherever two schedules must agree
+// bit for bit: which product of a b + c d is fused is otherwise the compiler's choice, made anew
+// in each kernel (the staged and the marching collision of the 16-bit formats fused ux^2 + uy^2
+// differently), and one last bit of FP32 flips the rounding of a stored 16-bit deviation.
 #pragma once
 
 #include "lattice.cuh"
@@ -12,6 +17,12 @@ template <>
 __device__ __forceinline__ double dev_log<double>(double x) { return log(x); }
 template <>
 __device__ __forceinline__ float dev_log<float>(float x) { return logf(x); }
+
+// a b and a - b, never fused with the operation around them
+__device__ __forceinline__ float mul_rn(float a, float b) { return __fmul_rn(a, b); }
+__device__ __forceinline__ double mul_rn(double a, double b) { return __dmul_rn(a, b); }
+__device__ __forceinline__ float sub_rn(float a, float b) { return __fsub_rn(a, b); }
+__device__ __forceinline__ double sub_rn(double a, double b) { return __dsub_rn(a, b); }
 
 // nu^s = mu^s/m^s - kappa lap rho^s - (1/3) ln rho^s for every component at one site
 // (Eq. lgf, Eq. chemicalpotential, Eq. definef).  The Flory-Huggins potential per
@@ -35,28 +46,27 @@ __device__ __forceinline__ void site_nu(const StepParams<C>& p, const C (&r)[N],
     for (int s = 0; s < N; ++s) phi[s] = r[s] * inv_rho;
     C sum_phi_m = C(0);
 #pragma unroll
-    for (int s = 0; s < N; ++s) sum_phi_m += phi[s] * p.inv_m[s];
+    for (int s = 0; s < N; ++s) sum_phi_m = fma(phi[s], p.inv_m[s], sum_phi_m);
     C chiphi[N];
     C quad = C(0);
 #pragma unroll
     for (int s = 0; s < N; ++s) {
         C acc = C(0);
 #pragma unroll
-        for (int t = 0; t < N; ++t) acc += p.chi[s * N + t] * phi[t];
+        for (int t = 0; t < N; ++t) acc = fma(p.chi[s * N + t], phi[t], acc);
         chiphi[s] = acc;
     }
 #pragma unroll
-    for (int s = 0; s < N; ++s) quad += C(0.5) * phi[s] * chiphi[s];
+    for (int s = 0; s < N; ++s) quad = fma(C(0.5) * phi[s], chiphi[s], quad);
     const C lnrho = dev_log(rho);
 #pragma unroll
     for (int s = 0; s < N; ++s) {
         C logs = -p.th_m[s] * lnrho;
         if (p.log_mask & (1u << s)) {
             const C fl = p.log_floor * rho;
-            logs += p.logc[s] * dev_log(r[s] > fl ? r[s] : fl);
+            logs = fma(p.logc[s], dev_log(r[s] > fl ? r[s] : fl), logs);
         }
-        const C bulk = p.theta * (p.m_inv_m1[s] - sum_phi_m + chiphi[s] - quad);
-        nu[s] = logs + bulk - p.kappa * lap[s];
+        nu[s] = fma(-p.kappa, lap[s], fma(p.theta, p.m_inv_m1[s] - sum_phi_m + chiphi[s] - quad, logs));
     }
 }
 
@@ -144,11 +154,11 @@ struct VDots {
 // (Sec. 3 equilibrium moments, all components built on the barycentric u).  The constant
 // w_i is added by collide() through its forcing bracket, so that 1 - 3/2 u.u is never
 // rounded: in FP32 that rounding has a sign set by u and changed the component masses
-// systematically (by up to 3e-8 of the density per step).
+// systematically (by up to 3e-8 of the density per step).  uu = u.u.
 template <typename C>
-__device__ __forceinline__ void eq_weights(C ux, C uy, C (&e)[Q])
+__device__ __forceinline__ void eq_weights(C ux, C uy, C uu, C (&e)[Q])
 {
-    const C base = C(-1.5) * (ux * ux + uy * uy);
+    const C base = C(-1.5) * uu;
     const VDots<C> du(ux, uy);
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
@@ -210,7 +220,7 @@ __device__ __forceinline__ void collide(const StepParams<C>& p, const C (&f)[Q],
     const VDots<C> da(ax, ay), dj(jx, jy);
     const C r3 = C(3) * r;
     const C omr = p.omega * r;
-    const C m3aj = fma(C(-3), ax * jx + ay * jy, omr - shift);
+    const C m3aj = fma(C(-3), fma(ax, jx, ay * jy), sub_rn(omr, shift));
     const C keep = C(1) - p.omega;
 #pragma unroll
     for (int i = 0; i < Q; ++i) {
@@ -219,6 +229,74 @@ __device__ __forceinline__ void collide(const StepParams<C>& p, const C (&f)[Q],
         out[i] = fma(keep, f[i], fma(omr, e[i], F));
     }
 }
+
+// ---------------------------------------------------------------- sums along a column
+//
+// The march (march.cuh) forms nu^s and its gradient from sums that it carries from row to row;
+// the tiles of the 16-bit formats (tile16.cuh) form the same sums at each site.  Stored with 8 or
+// 11 bits, the two agree only if every rounding does, so each sum stands here once.  Two choices keep
+// what the marches have always computed: FP32 with N = 1 has the other order in grad_rows, and
+// the batched march (APART) rounds theta times the sums over phi before it adds them.
+
+// What the nu^s of one site share: sum_t chi^{st} rho^t of every s, and the sums over phi
+template <typename C, int N, bool APART = false>
+struct SiteSums {
+    C acc[N], g;
+    __device__ __forceinline__ SiteSums(const StepParams<C>& p, const C (&r)[N], C inv)
+    {
+        C sm = C(0), quad = C(0);
+#pragma unroll
+        for (int t = 0; t < N; ++t) {
+            C a = C(0);
+#pragma unroll
+            for (int u = 0; u < N; ++u) a = fma(p.chi[t * N + u], r[u], a);
+            acc[t] = a;
+            sm = fma(r[t], p.inv_m[t], sm);
+            quad = fma(r[t], a, quad);
+        }
+        g = fma(sm, inv, C(0.5) * quad * inv * inv);
+    }
+    // nu^s without its gradient term
+    __device__ __forceinline__ C nu(const StepParams<C>& p, const C (&r)[N], C rho, C inv, C lnr, int s) const
+    {
+        C logs = -p.th_m[s] * lnr;
+        if ((p.log_mask >> s) & 1u) {
+            const C fl = p.log_floor * rho;
+            logs = fma(p.logc[s], dev_log(r[s] > fl ? r[s] : fl), logs);
+        }
+        const C own = fma(p.theta, fma(acc[s], inv, p.m_inv_m1[s]), logs);
+        return APART ? own + mul_rn(-p.theta, g) : fma(-p.theta, g, own);
+    }
+};
+
+// A row's parts of the Laplacian, from rho^s and A = rho^s(x - 1) + rho^s(x + 1):
+// 6 sum_i w_i (rho_i - rho_0) at row y is 6 (lap_side(y - 1) + lap_side(y + 1) + lap_mid(y))
+template <typename C>
+__device__ __forceinline__ C lap_side(C r, C A) { return fma(r, C(1.0 / 9.0), A * C(1.0 / 36.0)); }
+template <typename C>
+__device__ __forceinline__ C lap_mid(C r, C A) { return fma(A, C(1.0 / 9.0), -(C(5.0 / 9.0) * r)); }
+// nu^s of row y: without lap_side(y + 1), then whole.  k6 = 6 kappa, low = mul_rn(-k6, lap_side(y - 1))
+template <typename C>
+__device__ __forceinline__ C nu_part(C k6, C low, C nu0, C mid) { return fma(-k6, mid, low + nu0); }
+template <typename C>
+__device__ __forceinline__ C nu_whole(C k6, C part, C side) { return fma(-k6, side, part); }
+// The gradient over 3 at row y: d(y)/9 + (d(y - 1) + d(y + 1))/36 with d = nu(x + 1) - nu(x - 1), and
+// grad_rows(y + 1) - grad_rows(y - 1) with S = nu(x - 1) + nu(x + 1)
+template <typename C>
+__device__ __forceinline__ C grad_cols_part(C d, C d_below) { return fma(d, C(1.0 / 9.0), d_below * C(1.0 / 36.0)); }
+template <typename C>
+__device__ __forceinline__ C grad_cols(C part, C d_above) { return fma(d_above, C(1.0 / 36.0), part); }
+template <int N, typename C>
+__device__ __forceinline__ C grad_rows(C nu, C S)
+{
+    return N == 1 && sizeof(C) == 4 ? fma(S, C(1.0 / 36.0), nu * C(1.0 / 9.0)) : fma(nu, C(1.0 / 9.0), S * C(1.0 / 36.0));
+}
+// a^s from a third of grad nu^s (Eq. definef), g the body force
+template <typename C>
+__device__ __forceinline__ C accel_of(C fcoef, C third, C g) { return fma(-fcoef, C(3) * third, g); }
+// u.u
+template <typename C>
+__device__ __forceinline__ C speed2(C ux, C uy) { return fma(uy, uy, ux * ux); }
 
 // ---------------------------------------------------------------- component pairs
 //

@@ -38,7 +38,7 @@ __device__ __forceinline__ typename Storage<T>::C pull(const T* __restrict__ f,
         }
     }
     C v = Storage<T>::load(f + fidx(p, s, is, ys, xs));
-    if constexpr (Storage<T>::shifted) v += wq<C>(i) * __ldg(rho_line(f, p, s, ys) + p.hx + xs);
+    if constexpr (Storage<T>::shifted) v = fma(wq<C>(i), __ldg(rho_line(f, p, s, ys) + p.hx + xs), v);
     return v;
 }
 
@@ -130,22 +130,40 @@ k_density(const T* __restrict__ f, typename Storage<T>::C* __restrict__ rs,
         density_site<T, N, false>(f, rs, p, site, BAND ? nullptr : j);
 }
 
+// lap g = 6 sum_i w_i (g(r + v_i) - g(r)) and grad g = 3 sum_i w_i v_i g(r + v_i), from g0 = g(r) and
+// g(i) = g(r + v_i)
+template <typename C, typename G>
+__device__ __forceinline__ C laplacian_of(C g0, const G& g)
+{
+    C acc = C(0);
+#pragma unroll
+    for (int i = 1; i < Q; ++i) acc = fma(wq<C>(i), g(i) - g0, acc);
+    return C(6) * acc;
+}
+template <typename C, typename G>
+__device__ __forceinline__ void gradient_of(const G& g, C& gx, C& gy)
+{
+    C ax = C(0), ay = C(0);
+#pragma unroll
+    for (int i = 1; i < Q; ++i) {
+        const C v = g(i);
+        if (vx(i) != 0) ax = fma(wq<C>(i) * C(vx(i)), v, ax);
+        if (vy(i) != 0) ay = fma(wq<C>(i) * C(vy(i)), v, ay);
+    }
+    gx = C(3) * ax;
+    gy = C(3) * ay;
+}
+
 template <typename C, int N, bool E = true>
 __device__ __forceinline__ void neighbour_laplacians(const C* __restrict__ rs,
                                                      const StepParams<C>& p, int x, int y,
                                                      const C (&r)[N], C (&lap)[N])
 {
-    // lap g = 6 sum_i w_i (g(r + v_i) - g(r))
 #pragma unroll
-    for (int s = 0; s < N; ++s) {
-        C acc = C(0);
-#pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            const int xx = wrap_add(x, vx(i), p.nx), yy = stencil_row<E>(p, y, vy(i));
-            acc += wq<C>(i) * (rs[s * p.S + (long long)yy * p.nx + xx] - r[s]);
-        }
-        lap[s] = C(6) * acc;
-    }
+    for (int s = 0; s < N; ++s)
+        lap[s] = laplacian_of(r[s], [&](int i) {
+            return rs[s * p.S + (long long)stencil_row<E>(p, y, vy(i)) * p.nx + wrap_add(x, vx(i), p.nx)];
+        });
 }
 
 // nu^s at one site from the density fields.
@@ -185,16 +203,9 @@ template <bool E = true, typename C>
 __device__ __forceinline__ void field_grad(const C* __restrict__ g, const StepParams<C>& p, int x,
                                            int y, C& gx, C& gy)
 {
-    C ax = C(0), ay = C(0);
-#pragma unroll
-    for (int i = 0; i < Q; ++i) {
-        const int xx = wrap_add(x, vx(i), p.nx), yy = stencil_row<E>(p, y, vy(i));
-        const C v = g[(long long)yy * p.nx + xx];
-        ax += wq<C>(i) * C(vx(i)) * v;
-        ay += wq<C>(i) * C(vy(i)) * v;
-    }
-    gx = C(3) * ax;
-    gy = C(3) * ay;
+    gradient_of([&](int i) {
+        return g[(long long)stencil_row<E>(p, y, vy(i)) * p.nx + wrap_add(x, vx(i), p.nx)];
+    }, gx, gy);
 }
 
 // grad rho = 3 sum_i w_i v_i rho(r + v_i) of the total density, from the N density fields
@@ -227,8 +238,8 @@ __device__ __forceinline__ void site_accel(const C* __restrict__ rs, const C* __
     for (int s = 0; s < N; ++s) {
         C gx, gy;
         field_grad<E>(nu + s * p.S, p, x, y, gx, gy);
-        ax[s] = -p.fcoef * gx + p.gx;
-        ay[s] = -p.fcoef * gy + p.gy;
+        ax[s] = fma(-p.fcoef, gx, p.gx);
+        ay[s] = fma(-p.fcoef, gy, p.gy);
     }
     if (p.gd) {
         C grx, gry;
@@ -272,7 +283,7 @@ __device__ __forceinline__ void collide_site(const T* __restrict__ fin, T* __res
     const C inv = C(1) / rho;
     const C ux = jxt * inv, uy = jyt * inv;
     C e[Q];
-    eq_weights(ux, uy, e);
+    eq_weights(ux, uy, fma(ux, ux, uy * uy), e);
     C ax[N], ay[N];
     site_accel<C, N, E>(rs, nu, p, x, y, r, rho, ax, ay);
 #pragma unroll

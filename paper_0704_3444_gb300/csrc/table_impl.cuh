@@ -15,6 +15,7 @@
 #include "rows.cuh"
 #include "staged.cuh"
 #include "tile.cuh"
+#include "tile16.cuh"
 
 namespace mclb {
 
@@ -195,7 +196,10 @@ struct Launch {
     template <int N>
     static cudaError_t wall_tiles(const StepParams<C>& p, const T* fin, T* fout, cudaStream_t st)
     {
-        if constexpr (N * 32 * TILE_WALL_ROWS <= tile_max_threads<T>()) {
+        if constexpr (Storage<T>::shifted && N * 32 * TILE16_WALL_ROWS <= tile_max_threads<T>()) {
+            return launch_dependent(k_tile16_walls<T, N>, dim3((p.nx + 31) / 32, 2), N * 32 * TILE16_WALL_ROWS,
+                                    sizeof(C) * tile_smem_values(N, 32, TILE16_WALL_ROWS, false), st, fin, fout, p);
+        } else if constexpr (N * 32 * TILE_WALL_ROWS <= tile_max_threads<T>()) {
             return launch_dependent(k_tile_walls<T, N>, dim3((p.nx + 31) / 32, 2), N * 32 * TILE_WALL_ROWS,
                                     sizeof(C) * tile_smem_values(N, 32, TILE_WALL_ROWS, false), st, fin, fout, p);
         }
@@ -354,7 +358,9 @@ struct TileLaunch {
     //     512 x 384 x 3 14.7 / 18.5, 700 x 600 x 3 29.8 / 25.7; 400^2 x 4 21.7 / 20.1;
     //     300^2 x 5 13.5 / 19.4, 500 x 450 x 5 24.9 / 23.6; walls 1000 x 333 x 3 21 / 31,
     //     1500 x 1200 x 3 107 / 80.  k_tile, six and more: 300^2 x 6 20.0 / 23.1
-    //   16-bit: 400 x 300 x 4 19.7 / 22.8, 400^2 x 5 33 / 30; walls 1000 x 700 x 3 65.5 / 45.5
+    //   16-bit (k_tile16): 540^2 x 2 19.7 / 21.4, 440^2 x 3 20.7 / 22.1, 340^2 x 5 25.5 / 28.4, 270^2 x 8 31.1 /
+    //     41.8; walls (the march with its rows next to them by tiles) 510^2 x 3 27.9, 530^2 x 3 - / 30.0, 440^2
+    //     x 4 31.5, 460^2 x 4 - / 34.4, 390^2 x 5 33.8, 410^2 x 5 - / 40.2
     //   FP32 Gibbs-Duhem: 300^2 x 2 10.3 / 15.8, 512 x 384 x 3 22.8 / 18.5
     static long long most(const Problem& P)
     {
@@ -393,6 +399,8 @@ struct TileLaunch {
         pl.ty = ty;
         pl.gx = (P.nx + (1 << pl.lx) - 1) >> pl.lx;
         pl.gy = (P.ny + ty - 1) / ty;
+        if (Storage<T>::shifted && P.walls)   // the rows next to each wall are tiles of their own
+            pl.gy = P.ny <= TILE16_WALL_ROWS ? 1 : 2 + (std::max(0, P.ny - 2 * TILE16_WALL_ROWS) + ty - 1) / ty;
         pl.threads = P.N * (ty << pl.lx);
         pl.parts = 1;
         if (sizeof(C) == 8 && small && P.N <= 4) {   // a CTA of few warps: twice the threads
@@ -409,8 +417,8 @@ struct TileLaunch {
                             void* fout, cudaStream_t st)
     {
         const auto p = make_params<C>(P, sc.status);
-        const C* rs = nullptr;
-        if (P.force_form == FORCE_GIBBS_DUHEM) {
+        [[maybe_unused]] const C* rs = nullptr;
+        if (!Storage<T>::shifted && P.force_form == FORCE_GIBBS_DUHEM) {
             const cudaError_t e = launch_dependent(k_tile_rho<T>, dim3((unsigned)((P.S + 127) / 128), P.N),
                                                    128, 0, st, (const T*)fin, (C*)sc.rho_s, p);
             if (e != cudaSuccess) return e;
@@ -426,8 +434,13 @@ struct TileLaunch {
                 });
         }
         MCLB_DISPATCH_N(P.N, {
-            return launch_dependent(k_tile<T, NN>, dim3(pl.gx, pl.gy), pl.threads, pl.smem, st,
-                                    (const T*)fin, (T*)fout, rs, p, pl.lx, pl.ty, pl.parts);
+            if constexpr (Storage<T>::shifted)
+                return launch_dependent(P.walls ? k_tile16<T, NN, true> : k_tile16<T, NN, false>,
+                                        dim3(pl.gx, pl.gy), pl.threads, pl.smem, st, (const T*)fin, (T*)fout, p,
+                                        pl.lx, pl.ty);
+            else
+                return launch_dependent(k_tile<T, NN>, dim3(pl.gx, pl.gy), pl.threads, pl.smem, st,
+                                        (const T*)fin, (T*)fout, rs, p, pl.lx, pl.ty, pl.parts);
         });
     }
 };

@@ -13,10 +13,8 @@
 // What bounds it: on these lattices neither memory nor arithmetic but latency -- one round
 // trip to L2 for the pulls, two CTA barriers, one logarithm and one division, the launch.
 // The march spends (segment rows + 4) dependent row iterations on the same step and runs on
-// few SMs.
+// few SMs.  FP32 and FP64; the 16-bit formats have tile16.cuh.
 #pragma once
-
-#include <type_traits>
 
 #include "log64.cuh"
 #include "tma.cuh"
@@ -105,9 +103,9 @@ __device__ __forceinline__ C sum9(const C (&v)[Q])
 // operations fewer, the error of U on 64 x 64 FP64 grew from 2.2e-15 to 3.3e-15).
 template <typename C>
 __device__ __forceinline__ void collide_poly(const StepParams<C>& p, const C (&f)[Q], C r, C jx, C jy,
-                                             C ux, C uy, C ax, C ay, C shift, C (&out)[Q])
+                                             C ux, C uy, C ax, C ay, C (&out)[Q])
 {
-    const C omr = p.omega * r, keep = C(1) - p.omega, k0 = omr - shift;
+    const C omr = p.omega * r, keep = C(1) - p.omega;
     const C lx = C(3) * fma(omr, ux, r * ax), ly = C(3) * fma(omr, uy, r * ay);
     const C ax9 = C(9) * ax, ay9 = C(9) * ay;
     const C ou = C(4.5) * omr;
@@ -115,7 +113,7 @@ __device__ __forceinline__ void collide_poly(const StepParams<C>& p, const C (&f
     const C cxy = fma(C(2) * ou * ux, uy, fma(ax9, jy, ay9 * jx));
     const C tr = cxx + cyy, b = C(-1.0 / 3.0) * tr;
     const C w1 = wq<C>(1), w5 = wq<C>(5);
-    auto put = [&](int i, C g) { out[i] = fma(keep, f[i], fma(wq<C>(i), k0, g)); };
+    auto put = [&](int i, C g) { out[i] = fma(keep, f[i], fma(wq<C>(i), omr, g)); };
     put(0, wq<C>(0) * b);
     const C ex = w1 * (b + cxx), ey = w1 * (b + cyy), ox = w1 * lx, oy = w1 * ly;
     put(1, ex + ox);
@@ -366,29 +364,18 @@ __device__ __forceinline__ void tile_step(const T* __restrict__ fin, T* __restri
     const C ux = U[site], uy = U[SITES + site];
     C fjx, fjy, out[Q];
     forcing_momentum(p, r, jx, jy, ux, uy, fjx, fjy);
-    collide_poly(p, f, r, fjx, fjy, ux, uy, ax, ay, Storage<T>::shifted ? r : C(0), out);
+    collide_poly(p, f, r, fjx, fjy, ux, uy, ax, ay, out);
     // the new values, and their copies in the ghost columns where the tile touches an edge
     const bool edge = x0 < p.hx || x0 + TX > p.nx - p.hx;
     T* row = fout + (unsigned)(s * p.ny + y) * (Q * (unsigned)p.pitch);
-    auto put = [&](auto* line, C v) {
+    auto put = [&](T* line, C v) {
         if (edge)
             store_row(line, x, p.nx, p.hx, v);
         else
-            Storage<std::remove_pointer_t<decltype(line)>>::store(line + p.hx + x, v);
+            Storage<T>::store(line + p.hx + x, v);
     };
-    if constexpr (Storage<T>::shifted) {
-        C dsum = C(0);
 #pragma unroll
-        for (int i = 0; i < Q; ++i) {
-            const T d = Storage<T>::pack(out[i]);
-            dsum = add_wide<T>(dsum, d);
-            put(row + i * (unsigned)p.pitch, C(to_c<T>(d)));
-        }
-        put(rho_line(fout, p, s, y), r - dsum);
-    } else {
-#pragma unroll
-        for (int i = 0; i < Q; ++i) put(row + i * (unsigned)p.pitch, out[i]);
-    }
+    for (int i = 0; i < Q; ++i) put(row + i * (unsigned)p.pitch, out[i]);
 }
 
 // The three rows next to each wall (blockIdx.y: the lower, the upper one), for a lattice whose
