@@ -254,8 +254,9 @@ struct Launch {
         MCLB_DISPATCH_N(P.N, {
             // (few sites: smaller blocks, so that every SM has one)
             const int dt = P.S < 152LL * SITE_THREADS ? 64 : SITE_THREADS;
-            cudaError_t e = launch_dependent(k_density<T, NN, false>, dim3((unsigned)((P.S + dt - 1) / dt)), dt,
-                                             0, st, (const T*)f, (C*)sc.rho_s, p, U);
+            cudaError_t e = launch_dependent(U ? k_density<T, NN, false, true> : k_density<T, NN>,
+                                             dim3((unsigned)((P.S + dt - 1) / dt)), dt, 0, st, (const T*)f,
+                                             (C*)sc.rho_s, p, U);
             if (e != cudaSuccess) return e;
             return launch_dependent(k_fields<C, NN>, grid, 32 * warps, smem(rows), st, (const C*)sc.rho_s, rho,
                                     U, mu, Pt, p, rows);
