@@ -70,9 +70,11 @@ typedef enum {
 
 /* Which kernel schedule performs a timestep. */
 typedef enum {
-    MCLB_KERNEL_AUTO = 0,   /* the fused single-pass kernel, or on lattices too small to
-                               fill the GPU with it a kernel of small tiles (D2Q9, single
-                               handles): one launch per step, two with the Gibbs-Duhem form.
+    MCLB_KERNEL_AUTO = 0,   /* the fused single-pass kernel, or where it is faster a kernel of
+                               small tiles (D2Q9, single handles; lattices too small to fill
+                               the GPU with the other, and in FP64 every size but the larger
+                               ones of N = 4 and 5): one launch per step, two with the
+                               Gibbs-Duhem form.
                                In the 16-bit formats the state is that of FUSED bit for bit,
                                whichever AUTO picks                                */
     MCLB_KERNEL_FUSED = 1,  /* stream, moments, potentials, force, collision in one

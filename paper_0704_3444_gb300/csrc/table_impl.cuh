@@ -352,13 +352,17 @@ struct TileLaunch {
     // Most sites x components for which a tile kernel beats the march (measured on both sides of
     // each line, us per step, tile / march; between walls the march has one launch more):
     //   FP64: it runs at the FP64 pipe's rate on every SM with fewer FP64 instructions a site:
-    //     64 x 64 x 2 9.73 / 107, 2048^2 x 2 2323 / 2613, 2048^2 x 3 3474 / 3802, 600^2 x 6 758 /
-    //     1233, 500^2 x 8 714 / 1130, Gibbs-Duhem 1024^2 x 3 967 / 1132: every size, but
-    //     1024^2 x 4 1270 / 1230, 1024^2 x 5 1640 / 1494
+    //     64 x 64 x 2 5.3 / 107, 2048^2 x 2 2323 / 2613, 2048^2 x 3 3474 / 3802, 500^2 x 6 533 / 850, 1700^2
+    //     x 6 6110 / 10642, x 7 7247 / 12506, x 8 8172 / 14210, Gibbs-Duhem 900^2 x 3 728 / 869: every
+    //     size, but 700^2 x 4 610 / 621, 860^2 x 4 912 / 901 and 500^2 x 5 399 / 415, 700^2 x 5 777 /
+    //     757; walls 700^2 x 4 609 / 646, 850^2 x 4 906 / 906, 700^2 x 5 778 / 783
     //   FP32 (k_rows): 1000^2 x 1 18.1 / 26.3; 700^2 x 2 20.5 / 22.3, 1024^2 x 2 38 / 37;
     //     512 x 384 x 3 14.7 / 18.5, 700 x 600 x 3 29.8 / 25.7; 400^2 x 4 21.7 / 20.1;
-    //     300^2 x 5 13.5 / 19.4, 500 x 450 x 5 24.9 / 23.6; walls 1000 x 333 x 3 21 / 31,
-    //     1500 x 1200 x 3 107 / 80.  k_tile, six and more: 300^2 x 6 20.0 / 23.1
+    //     300^2 x 5 13.5 / 19.4, 500 x 450 x 5 24.9 / 23.6.  k_tile, six and more: 300^2 x 6 20.0 / 23.1
+    //   FP32 between walls (the march with its rows next to them by tiles): 1500^2 x 1 42 / 57; 800^2 x 2
+    //     26.2 / 31.4, 1000^2 x 2 39.4 / 38.7; 800^2 x 3 39.0 / 40.5; 600^2 x 4 33.3 / 33.8, 700^2 x 4 43.2 /
+    //     41.1; 500^2 x 5 29.3 / 30.2, 600^2 x 5 42.4 / 38.6; 350^2 x 6 26.4 / 29.2, 400^2 x 6 33.1 / 33.0;
+    //     350^2 x 7 31.5 / 32.4, 400^2 x 7 40.0 / 37.3; 300^2 x 8 28.6 / 33.7, 350^2 x 8 37.7 / 34.3
     //   16-bit (k_tile16): 540^2 x 2 19.7 / 21.4, 440^2 x 3 20.7 / 22.1, 340^2 x 5 25.5 / 28.4, 270^2 x 8 31.1 /
     //     41.8; walls (the march with its rows next to them by tiles) 510^2 x 3 27.9, 530^2 x 3 - / 30.0, 440^2
     //     x 4 31.5, 460^2 x 4 - / 34.4, 390^2 x 5 33.8, 410^2 x 5 - / 40.2
@@ -366,10 +370,17 @@ struct TileLaunch {
     static long long most(const Problem& P)
     {
         const int N = P.N;
-        if (sizeof(C) == 8) return N == 4 || N == 5 ? 3000000 : 1LL << 40;
+        if (sizeof(C) == 8) {
+            if (N == 4) return P.walls ? 2900000 : 2400000;
+            if (N == 5) return P.walls ? 2500000 : 1800000;
+            return 1LL << 40;
+        }
         if (P.force_form == FORCE_GIBBS_DUHEM) return 350000;
         if (Storage<T>::shifted) return P.walls ? 800000 : 600000;
-        if (P.walls) return 2500000;
+        if (P.walls) {
+            constexpr int by_n[NMAX] = {2500000, 1900000, 2200000, 1500000, 1300000, 950000, 900000, 800000};
+            return by_n[N - 1];
+        }
         return N == 1 ? 2000000 : N == 2 ? 1200000 : N == 4 || N >= 6 ? 550000 : 900000;
     }
 

@@ -236,3 +236,19 @@ def test_16_bit_schedules_agree(shape, precision):
     assert auto[3] < fused[3]
     for a, b in zip(auto[:3], fused[:3]):
         assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("precision,shape,walls,launches", [
+    ("fp64", (690, 700, 4), 0, 1), ("fp64", (800, 800, 4), 0, 2), ("fp64", (560, 560, 5), 0, 1),
+    ("fp64", (770, 770, 5), 0, 2), ("fp64", (700, 690, 5), 1, 1), ("fp64", (760, 760, 5), 1, 3),
+    ("fp64", (900, 900, 6), 0, 1), ("fp32", (1500, 1500, 1), 1, 1), ("fp32", (1050, 1050, 2), 1, 3),
+    ("fp32", (800, 800, 3), 1, 1), ("fp32", (785, 785, 4), 1, 3), ("fp32", (700, 700, 5), 1, 3),
+    ("fp32", (300, 350, 6), 1, 1), ("fp32", (500, 500, 6), 1, 3), ("fp32", (400, 400, 7), 1, 3),
+    ("fp32", (300, 300, 8), 1, 1), ("fp32", (400, 400, 8), 1, 3)], ids=str)
+def test_auto_takes_the_faster_schedule(precision, shape, walls, launches):
+    """On both sides of the lines where tiles and march measured equal: one launch a step is the
+    tiles, two (three between walls) the march."""
+    nx, ny, n = shape
+    sim = mclb.Simulation(n, nx, ny, 0.9, inputs.uniform_chi(n, 1.6), precision=precision, walls=walls)
+    assert sim.launches_per_step == launches
+    sim.close()
