@@ -126,8 +126,8 @@ typedef enum {
                         over z planes that forms the potentials on chip and collides (two
                         launches per step; N <= 4, Eq. definef as printed; FUSED fails
                         with MCLB_EINVAL otherwise, AUTO falls back, and takes it only
-                        where it is the faster one: FP32, N <= 3, from about 1e6
-                        site-components on); STAGED: three launches.  The two schedules give the same values bit for bit.
+                        where it is the faster one: FP32 from about 1e6
+                        site-components on, N = 1 and 4 from 8.5e6 and 6.2e6); STAGED: three launches.  The two schedules give the same values bit for bit.
                         Fields are [.][z][y][x]; U has 3 components, P 6 (xx, xy, xz, yy,
                         yz, zz), the momentum and force sums 3                             */
 } mclb_lattice;

@@ -811,12 +811,17 @@ struct Launch19 {
             return 1;
         }
     }
-    // The march pays up to three components from about 1e6 site-components on (us per step, march
-    // / staged: 192^3 x 3 895 / 1056, 100 x 90 x 70 x 2 66 / 73, 128 x 120 x 100 x 4 311 / 311; 64 x
-    // 60 x 50 x 3 50 / 28, 40 x 24 x 30 x 3 37 / 10: too few CTAs, each with its dependent plane
-    // iterations), and not in FP64, which the FP64 pipe bounds and whose pulled values spill
-    // (64^3 x 3 877 / 355, 128 x 128 x 96 x 2 2477 / 1396).
-    static bool pays(const Problem& P) { return sizeof(C) == 4 && P.N <= 3 && P.S * P.N >= 1200000; }
+    // The march pays in FP32 from a number of site-components on, below which its CTAs are too few, each
+    // with its dependent plane iterations (us per step, march / staged: 192^3 x 1 390 / 382, 224^3 x 1
+    // 578 / 603; 100 x 90 x 70 x 2 66 / 73, 192^3 x 2 627 / 723; 40 x 24 x 30 x 3 37 / 10, 64^3 x 3 53 / 42,
+    // 96^3 x 3 131 / 140, 192^3 x 3 873 / 1055; 96^3 x 4 189 / 184, 128 x 120 x 100 x 4 311 / 311, 128^3 x 4
+    // 406 / 419, 192^3 x 4 1310 / 1418), and not in FP64, which the FP64 pipe bounds and whose pulled
+    // values spill (64^3 x 3 1063 / 357, 128^3 x 4 6082 / 3547).
+    static bool pays(const Problem& P)
+    {
+        const long long least = P.N == 1 ? 8500000 : P.N == 4 ? 6200000 : 1200000;
+        return sizeof(C) == 4 && P.N <= M3_NMAX && P.S * P.N >= least;
+    }
 
     static int plan(Problem& P, int sm_count)
     {

@@ -252,3 +252,27 @@ def test_auto_takes_the_faster_schedule(precision, shape, walls, launches):
     sim = mclb.Simulation(n, nx, ny, 0.9, inputs.uniform_chi(n, 1.6), precision=precision, walls=walls)
     assert sim.launches_per_step == launches
     sim.close()
+
+
+@pytest.mark.parametrize("n,edge,launches", [(1, 128, 3), (1, 224, 2), (2, 96, 2), (4, 96, 3), (4, 128, 2)])
+def test_auto_takes_the_faster_d3q19_schedule(n, edge, launches):
+    """As above: three launches a step are the staged step, two the march; the fields are those of
+    the other schedule bit for bit."""
+    import torch
+    rho = 1.0 / n + 0.02 * torch.rand(n, edge, edge, edge, generator=torch.Generator("cuda").manual_seed(n),
+                                      dtype=torch.float64, device="cuda")
+    u = torch.zeros(3, edge, edge, edge, dtype=torch.float64, device="cuda")
+    got = []
+    for kernel in (mclb.KERNEL_AUTO, mclb.KERNEL_STAGED if launches == 2 else mclb.KERNEL_FUSED):
+        sim = mclb.Simulation(n, edge, edge, 0.9, inputs.uniform_chi(n, 1.6), precision="fp32", lattice="d3q19",
+                              nz=edge, kappa=0.02, kernel=kernel)
+        assert sim.launches_per_step == (launches if kernel == mclb.KERNEL_AUTO else 5 - launches)
+        r, v = rho.clone(), u.clone()
+        sim.init_fields_device(r, v)
+        torch.cuda.synchronize()
+        sim.step(3)
+        sim.moments_device(rho=r, U=v)
+        assert sim.status() == 0
+        got.append((r.cpu(), v.cpu()))
+        sim.close()
+    assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
