@@ -308,9 +308,20 @@ k19_density(const T* __restrict__ f, typename Storage<T>::C* __restrict__ rs,
         }
 }
 
+// The Laplacian of lap19 difference by difference, for the output mu^s: the sums of lap19 cancel
+// against 4 g(r), which at kappa = 0.5 made the error of an FP32 mu^s 8 % larger (1.55e-7 -> 1.68e-7).
+template <typename C, typename G>
+__device__ __forceinline__ C lap19_by_differences(C g0, const G& g)
+{
+    C acc = C(0);
+#pragma unroll
+    for (int i = 1; i < Q19; ++i) acc = fma(w19<C>(i), g(i) - g0, acc);
+    return C(6) * acc;
+}
+
 // lap g = 6 sum_i w_i (g(r + v_i) - g(r)) of every component's density field (each
 // neighbour's index formed once for all components).
-template <typename C, int N>
+template <typename C, int N, bool DIFF = false>
 __device__ __forceinline__ void laplacians19(const C* __restrict__ rs, const StepParams<C>& p,
                                              const Site3& c, const C (&r)[N], C (&lap)[N])
 {
@@ -323,7 +334,10 @@ __device__ __forceinline__ void laplacians19(const C* __restrict__ rs, const Ste
         for (int s = 0; s < N; ++s) g[s][i] = rs[s * p.S + t];
     }
 #pragma unroll
-    for (int s = 0; s < N; ++s) lap[s] = lap19(r[s], [&](int i) { return g[s][i]; });
+    for (int s = 0; s < N; ++s) {
+        auto at = [&](int i) { return g[s][i]; };
+        lap[s] = DIFF ? lap19_by_differences(r[s], at) : lap19(r[s], at);
+    }
 }
 
 template <typename C, int N>
@@ -574,7 +588,7 @@ k19_moments(const C* __restrict__ rs, const C* __restrict__ nu, double* __restri
     }
     if (mu_out || P) {
         C lap[N], mu[N];
-        laplacians19<C, N>(rs, p, c, r, lap);
+        laplacians19<C, N, true>(rs, p, c, r, lap);
         site_mu<C, N>(p, r, lap, mu);
         if (mu_out)
 #pragma unroll

@@ -6,8 +6,10 @@
 // issue (FP32 output widened to FP64 by moving bits: the conversion instruction runs in the
 // FP64 pipe).  Before, nu^s went through memory in a launch of its own, bound by the index
 // arithmetic of its neighbour loads, and the output pass pulled every population again for
-// the momentum.  us a call, before / now: 8192 x 2048 x 3 FP32 1158 / 662, 2048^2 x 5 FP32 523 / 314,
-// BF16 750 / 391, 64 x 64 x 2 FP64 38 / 20.
+// the momentum.  The Laplacian is summed from differences of neighbours: by sums that cancel against
+// 10/3 rho^s the error of an FP32 mu^s grew by a quarter at kappa = 0.5 (1.13e-7 -> 1.41e-7).
+// us a call (rho, U, mu), before / now: 8192 x 2048 x 3 FP32 1386 / 814, 2048^2 x 5 FP32 543 / 329,
+// BF16 778 / 401, 64 x 64 x 2 FP64 40 / 18, 2048^2 x 2 FP64 3141 / 2894.
 #pragma once
 
 #include "staged.cuh"
@@ -51,10 +53,8 @@ k_fields(const C* __restrict__ rs, double* __restrict__ rho_out, double* __restr
     }
     __syncthreads();
 
-    auto laplacian = [&](const C* g, int up, int dn) {   // 6 sum_i w_i (g(r + v_i) - g(r))
-        const C ax = (g[-1] + g[1]) + (g[up] + g[dn]);
-        const C di = (g[up - 1] + g[up + 1]) + (g[dn - 1] + g[dn + 1]);
-        return fma(C(2.0 / 3.0), ax, fma(C(1.0 / 6.0), di, C(-10.0 / 3.0) * g[0]));
+    auto laplacian = [&](const C* g, int up, int dn) {
+        return laplacian_of(g[0], [&](int i) { return g[(vy(i) < 0 ? up : vy(i) > 0 ? dn : 0) + vx(i)]; });
     };
     auto gradient = [&](const C* g, int up, int dn, C& gx, C& gy) {   // 3 sum_i w_i v_i g(r + v_i)
         const C ne = g[dn + 1], nw = g[dn - 1], se = g[up + 1], sw = g[up - 1];

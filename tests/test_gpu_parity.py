@@ -507,3 +507,37 @@ def test_n5_spinodal_per_field():
             assert np.abs(g[k] - ref500[k]).max() < b, (prec, k)
         assert np.abs(g["P"] - ref500["P"]).max() < bp, prec
         sim.close()
+
+
+@pytest.mark.parametrize("lattice", ["d2q9", "d3q19"])
+def test_mu_of_a_smooth_field_at_large_kappa(lattice):
+    """mu^s of an FP32 state against the definition in FP64 on the state's own rho^s, kappa = 50 on a
+    field of long waves: the Laplacian has to come from differences of neighbours, which are
+    exact here.  Sums that cancel against 4 rho are off by kappa times a rounding of 4 rho,
+    50 x 1.2e-7; the other terms of mu are about ten roundings of values below 1.5, under 2e-6
+    together."""
+    n, nx, ny, nz = 2, 120, 90, 4 if lattice == "d3q19" else 1
+    x = 2 * np.pi * np.arange(nx)[None, None, :] / nx
+    y = 2 * np.pi * np.arange(ny)[None, :, None] / ny
+    wave = 0.1 * np.sin(x) * np.cos(y) + np.zeros((nz, 1, 1))
+    rho = np.stack([0.6 + wave, 0.4 - wave])
+    if nz == 1:
+        rho = rho[:, 0]
+    chi = inputs.uniform_chi(n, 1.5)
+    sim = mclb.Simulation(n, nx, ny, 1.0, chi, precision="fp32", kappa=50.0, lattice=lattice,
+                          **({"nz": nz} if nz > 1 else {}))
+    sim.init_fields(rho)
+    m = sim.moments()
+    sim.close()
+    r = m["rho"].reshape(n, nz, ny, nx)
+    phi = r / r.sum(0)
+    chiphi = np.einsum("st,tzyx->szyx", chi, phi)
+    w = {1: 1 / 9, 2: 1 / 36} if lattice == "d2q9" else {1: 1 / 18, 2: 1 / 36}
+    lap = np.zeros_like(r)
+    for c in np.ndindex(3, 3, 3):
+        c = tuple(v - 1 for v in c)
+        k = sum(abs(v) for v in c)
+        if k in w and (nz > 1 or c[0] == 0):
+            lap += 6 * w[k] * (np.roll(r, c, (1, 2, 3)) - r)
+    mu = (np.log(phi) + 1 - 1 - phi.sum(0) + chiphi - 0.5 * (phi * chiphi).sum(0)) / 3 - 50.0 * lap
+    assert np.max(np.abs(m["mu"] - mu.reshape(m["mu"].shape))) < 2e-6
