@@ -541,3 +541,30 @@ def test_mu_of_a_smooth_field_at_large_kappa(lattice):
             lap += 6 * w[k] * (np.roll(r, c, (1, 2, 3)) - r)
     mu = (np.log(phi) + 1 - 1 - phi.sum(0) + chiphi - 0.5 * (phi * chiphi).sum(0)) / 3 - 50.0 * lap
     assert np.max(np.abs(m["mu"] - mu.reshape(m["mu"].shape))) < 2e-6
+
+
+@pytest.mark.parametrize("lattice", ["d2q9", "d3q19"])
+def test_fp32_fields_widen_exactly(lattice):
+    """rho of an FP32 state as the output fields hand it out in FP64 is the float itself: every
+    exponent, fractions at their ends, both signs, subnormals, zero, infinities and NaN (set as one
+    population, the others zero; values beyond FP32 become infinite, two of opposite sign NaN)."""
+    frac = np.array([0, 1, 2, 0x155555, 0x400000, 0x7FFFFE, 0x7FFFFF], dtype=np.uint32)
+    bits = (np.arange(255, dtype=np.uint32)[:, None] << 23 | frac).ravel()
+    v = bits.view(np.float32).astype(np.float64)
+    v = np.concatenate([v, -v, [1e39, -1e39, 1e39]])
+    nx, nz = 60, 3 if lattice == "d3q19" else 1
+    ny = -(-v.size // (nx * nz))
+    v = np.concatenate([v, np.ones(nx * ny * nz - v.size)])
+    last = 2 * bits.size + 2                    # the site that gets both signs
+    f = np.zeros((1, 19 if nz > 1 else 9, nx * ny * nz))
+    f[0, 0] = v
+    f[0, 1, last] = -1e39
+    sim = mclb.Simulation(1, nx, ny, 1.0, [[0.0]], precision="fp32", lattice=lattice, **({"nz": nz} if nz > 1 else {}))
+    sim.set_state(f.reshape((1, -1, nz, ny, nx) if nz > 1 else (1, -1, ny, nx)))
+    got = sim.moments(U=False, mu=False, P=False)["rho"].ravel()
+    sim.close()
+    with np.errstate(over="ignore"):
+        want = v.astype(np.float32).astype(np.float64)
+    assert np.isnan(got[last])
+    got[last] = want[last] = 0.0
+    assert np.array_equal(got, want)
