@@ -276,3 +276,30 @@ def test_auto_takes_the_faster_d3q19_schedule(n, edge, launches):
         got.append((r.cpu(), v.cpu()))
         sim.close()
     assert torch.equal(got[0][0], got[1][0]) and torch.equal(got[0][1], got[1][1])
+
+
+@pytest.mark.parametrize("n,sizes", [
+    (1, [(160, 97), (1, 1), (33, 40)]), (2, [(128, 104), (130, 61), (17, 9)]), (3, [(16, 8), (121, 113), (5, 3)]),
+    (6, [(64, 48), (67, 35), (4, 9)]), (8, [(24, 12), (41, 30)])], ids=lambda v: str(v) if isinstance(v, int) else "")
+def test_fp64_batch_by_tiles(n, sizes):
+    """FP64 batches by tiles of 16 x 8 (more than 12800 sites in all) and of 8 x 4 sites (five and more
+    components), exact multiples and remainders: every state within 1e-12 of the oracle after a
+    replayed graph of 32 steps and nine more."""
+    probs = []
+    for k, (nx, ny) in enumerate(sizes):
+        rho, u = inputs.random_state(n, nx, ny, seed=680 + k, amp=0.3, umax=0.02)
+        p = inputs.Problem(name=f"f{k}", ncomp=n, nx=nx, ny=ny, tau=0.8 + 0.1 * k, chi=inputs.uniform_chi(n, 1.6),
+                           m=np.array([1.0 + (s % 3) for s in range(n)]), theta=0.4, kappa=0.02, force=(1e-5, -2e-5),
+                           rho=rho, u=u)
+        p.forcing_velocity = k % 2
+        probs.append(p)
+    b = mclb.Batch(probs, precision="fp64")
+    b.init_all()
+    b.step(41)
+    assert [w for _, w in b.tuning()] == [1] and b.launches_per_step == 2
+    assert b.status()[0] == 0
+    for k, p in enumerate(probs):
+        orc = Oracle.from_problem(p)
+        assert orc.run(41) == 0
+        assert _rel(b.get_state(k), orc.f) < 1e-12, k
+    b.close()
