@@ -392,7 +392,7 @@ struct TileLaunch {
     {
         TilePlan pl{};
         const bool gd = P.force_form == FORCE_GIBBS_DUHEM;
-        if (P.S * P.N > most(P)) return pl;
+        if (P.S * P.N > most(P) || (gd && (Storage<T>::shifted || P.N > TILE_GD_NMAX))) return pl;
         if constexpr (std::is_same<T, float>::value) {
             if (!gd && P.S * P.N >= ROWS_LEAST && P.ny >= ROWS_MIN_NY && P.N <= ROWS_NMAX) {
                 pl.gx = (P.nx + ROWS_X - 1) / ROWS_X;
@@ -430,11 +430,13 @@ struct TileLaunch {
     {
         const auto p = make_params<C>(P, sc.status);
         [[maybe_unused]] const C* rs = nullptr;
-        if (!Storage<T>::shifted && P.force_form == FORCE_GIBBS_DUHEM) {
-            const cudaError_t e = launch_dependent(k_tile_rho<T>, dim3((unsigned)((P.S + 127) / 128), P.N),
-                                                   128, 0, st, (const T*)fin, (C*)sc.rho_s, p);
-            if (e != cudaSuccess) return e;
-            rs = (const C*)sc.rho_s;
+        if constexpr (!Storage<T>::shifted) {
+            if (P.force_form == FORCE_GIBBS_DUHEM) {
+                const cudaError_t e = launch_dependent(k_tile_rho<T>, dim3((unsigned)((P.S + 127) / 128), P.N),
+                                                       128, 0, st, (const T*)fin, (C*)sc.rho_s, p);
+                if (e != cudaSuccess) return e;
+                rs = (const C*)sc.rho_s;
+            }
         }
         if constexpr (std::is_same<T, float>::value) {
             if (pl.lx == 0)

@@ -30,6 +30,9 @@ constexpr int tile_max_threads() { return sizeof(typename Storage<T>::C) == 8 ? 
 template <typename T>
 constexpr int tile_max_regs(int n) { return sizeof(typename Storage<T>::C) == 8 ? (n <= 4 ? 80 : 128) : 56; }
 
+// Components up to which the tiles have the Gibbs-Duhem form (as the march, whose place they take)
+constexpr int TILE_GD_NMAX = 3;
+
 // Shared memory of one CTA in values of C: rho^s, nu^s, j^s, u and (Gibbs-Duhem) rho, 1/rho, a^s.
 __host__ __device__ constexpr int tile_smem_values(int n, int tx, int ty, bool gd)
 {
@@ -199,6 +202,7 @@ __device__ __forceinline__ void tile_step(const T* __restrict__ fin, T* __restri
     using C = typename Storage<T>::C;
     constexpr bool F64 = sizeof(C) == 8;
     const int parts = F64 ? parts64 : 1;
+    const bool gd = N <= TILE_GD_NMAX && p.gd;
     __shared__ Log64Row tab[F64 ? LOG64_ROWS : 1];
     extern __shared__ __align__(16) unsigned char tile_raw[];
     const int TX = 1 << lx, SITES = ty << lx;
@@ -310,7 +314,7 @@ __device__ __forceinline__ void tile_step(const T* __restrict__ fin, T* __restri
             NU[(t * NY + by) * NX + bx] = nu[t];
         }
         if (part != parts - 1) continue;
-        if (p.gd) RT[by * NX + bx] = rho;
+        if (gd) RT[by * NX + bx] = rho;
         if (k < SITES) {
             C ux = C(0), uy = C(0);
 #pragma unroll
@@ -320,7 +324,7 @@ __device__ __forceinline__ void tile_step(const T* __restrict__ fin, T* __restri
             }
             U[k] = ux * inv;
             U[SITES + k] = uy * inv;
-            if (p.gd) IT[k] = inv;
+            if (gd) IT[k] = inv;
             if (x0 + bx - 1 < p.nx && yy < p.ny && (!(rho > C(0)) || !isfinite(rho)))
                 atomicOr(p.status, STATUS_NONFINITE);
         }
@@ -340,7 +344,7 @@ __device__ __forceinline__ void tile_step(const T* __restrict__ fin, T* __restri
         ax = fma(-p.fcoef, ax, p.gx);
         ay = fma(-p.fcoef, ay, p.gy);
     }
-    if (p.gd) {
+    if (gd) {
         // the common shift (A_c - A)/rho of every component (gibbs_duhem_shift)
         if (mine) {
             A[s * SITES + site] = ax - p.gx;
