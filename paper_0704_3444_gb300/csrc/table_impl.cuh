@@ -352,7 +352,7 @@ struct TileLaunch {
     // Most sites x components for which a tile kernel beats the march (measured on both sides of
     // each line, us per step, tile / march; between walls the march has one launch more):
     //   FP64: it runs at the FP64 pipe's rate on every SM with fewer FP64 instructions a site:
-    //     64 x 64 x 2 5.3 / 107, 2048^2 x 2 2323 / 2613, 2048^2 x 3 3474 / 3802, 500^2 x 6 533 / 850, 1700^2
+    //     64 x 64 x 2 9.65 / 107, 2048^2 x 2 2323 / 2613, 2048^2 x 3 3474 / 3802, 500^2 x 6 533 / 850, 1700^2
     //     x 6 6110 / 10642, x 7 7247 / 12506, x 8 8172 / 14210, Gibbs-Duhem 900^2 x 3 728 / 869: every
     //     size, but 700^2 x 4 610 / 621, 860^2 x 4 912 / 901 and 500^2 x 5 399 / 415, 700^2 x 5 777 /
     //     757; walls 700^2 x 4 609 / 646, 850^2 x 4 906 / 906, 700^2 x 5 778 / 783

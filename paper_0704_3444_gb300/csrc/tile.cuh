@@ -202,7 +202,6 @@ __device__ __forceinline__ void tile_step(const T* __restrict__ fin, T* __restri
     using C = typename Storage<T>::C;
     constexpr bool F64 = sizeof(C) == 8;
     const int parts = F64 ? parts64 : 1;
-    const bool gd = N <= TILE_GD_NMAX && p.gd;
     __shared__ Log64Row tab[F64 ? LOG64_ROWS : 1];
     extern __shared__ __align__(16) unsigned char tile_raw[];
     const int TX = 1 << lx, SITES = ty << lx;
@@ -314,7 +313,7 @@ __device__ __forceinline__ void tile_step(const T* __restrict__ fin, T* __restri
             NU[(t * NY + by) * NX + bx] = nu[t];
         }
         if (part != parts - 1) continue;
-        if (gd) RT[by * NX + bx] = rho;
+        if (N <= TILE_GD_NMAX && p.gd) RT[by * NX + bx] = rho;
         if (k < SITES) {
             C ux = C(0), uy = C(0);
 #pragma unroll
@@ -324,7 +323,7 @@ __device__ __forceinline__ void tile_step(const T* __restrict__ fin, T* __restri
             }
             U[k] = ux * inv;
             U[SITES + k] = uy * inv;
-            if (gd) IT[k] = inv;
+            if (N <= TILE_GD_NMAX && p.gd) IT[k] = inv;
             if (x0 + bx - 1 < p.nx && yy < p.ny && (!(rho > C(0)) || !isfinite(rho)))
                 atomicOr(p.status, STATUS_NONFINITE);
         }
@@ -344,7 +343,7 @@ __device__ __forceinline__ void tile_step(const T* __restrict__ fin, T* __restri
         ax = fma(-p.fcoef, ax, p.gx);
         ay = fma(-p.fcoef, ay, p.gy);
     }
-    if (gd) {
+    if (N <= TILE_GD_NMAX && p.gd) {
         // the common shift (A_c - A)/rho of every component (gibbs_duhem_shift)
         if (mine) {
             A[s * SITES + site] = ax - p.gx;
