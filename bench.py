@@ -342,7 +342,8 @@ def run_lines(torch, mclb, sptr, stream, count=512, nx=1024, steps=4096, precisi
            "precision": precision,
            "launches_per_step_chunk": b.launches_per_step, "status_ok": rc == 0,
            "note": f"MLUPS x N of {count} D1Q3 lines advanced {steps} steps by one resident "
-                   "launch (one CTA per line, the line in shared memory): bound by the "
+                   "launch (one CTA per line, in FP64 up to a cluster of eight; the line in "
+                   "shared memory): bound by the "
                    "per-site arithmetic (FP64 runs at a small fraction of the FP32 rate on "
                    "this GPU), not by HBM"}
     b.close()

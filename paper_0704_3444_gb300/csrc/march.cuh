@@ -149,7 +149,7 @@ __device__ __forceinline__ void march_cta(const CUtensorMap* tmap, const CUtenso
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     // rows whose density the status word checks: with walls, the three rows next to each
     // wall are written here with periodic neighbours and then rewritten by the wall-aware
-    // staged launches, so only those launches check them
+    // launches (tiles, or the staged bands), so only those check them
     const int ychk0 = p.walls ? max(y0, 3) : y0;
     const int ychk1 = p.walls ? min(y0 + Hc, p.ny - 3) : y0 + Hc;
 

@@ -10,8 +10,11 @@
 // around) and u, barrier, collision, store with ghost columns.
 //
 // Populations read per written one: 12 x 32 / (8 x 28) = 1.71, the surplus from L2.  What
-// bounds it is the issue rate with all rows of the lattice in flight at once; the march
-// needs segment rows + 4 dependent iterations of about 1.2 us for the same step.  Eight rows: with
+// bounds it is the chain of one step (pull from L2, barrier, logarithm and division, barrier,
+// store, next launch) and, the more tiles there are, instruction issue: about 740 instructions a
+// warp, issue slots 43 % busy at 256^2 x 3 (0.7 of a wave of CTAs), 56 % at 512 x 384 x 3, 64 % at 1000 x 333
+// x 3 between walls.  The march needs segment rows + 4 dependent iterations of about 1.2 us for
+// the same step.  Eight rows: with
 // 10 or 12, which pull 1.4 and 1.33 rows for each written one, CTAs are larger and fewer (us per
 // step, 8 / 10 / 12 rows: 256^2 x 3 8.85 / 8.62 / 9.27, 300^2 x 2 8.0 / 8.5 / 8.8, 512 x 384 x 3 14.3 /
 // 14.5 / 15.3, 700^2 x 2 18.8 / 20.3 / 19.8; 48 batched instances 153 / - / 184).  (The pulls by
